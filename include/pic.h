@@ -410,8 +410,9 @@ pic_status pic_use_graphs(pic_ctx *c, int enable);
 /* Launch-shape autotuner (default off).  enable = 1: whenever a pic_step
  * call meets tier-0 staging sizes whose tuning is not finished, its first
  * steps run the cell kernel with 1, 2, 4 and 8 warps per CTA (as many as fit
- * in shared memory), each twice in the order 1 2 4 8 8 4 2 1, timing the
- * cell kernels with CUDA events; the fastest mean is kept for those sizes.
+ * in shared memory; 4 alone where a cell takes a team of four), each twice
+ * in the order 1 2 4 8 8 4 2 1, timing the cell kernels with CUDA events; the
+ * fastest mean is kept for those sizes.
  * The context's first step is not timed.  These are steps of the
  * simulation: the launch shape changes no result.  enable = 0 stops tuning
  * (choices made are kept); -1 leaves it as is.  wpc_out (may be NULL) gets
@@ -446,9 +447,9 @@ pic_status pic_dd_sum_check(const float *x, int n, double *out);
 
 /* The in-cell ordering of the device (ascending key, ties by id; the
  * canonical order every per-cell rule follows), run on n <= 4096 given
- * entries by one warp with the algorithm a cell of that size uses in the
- * cell-kernel instance rmax (128, 512 or 1024: the largest cell it sorts in
- * registers; the radix sort above 512, resp. 1024; rmax 128 takes n <= 128):
+ * entries with the algorithm a cell of that size uses in the cell-kernel
+ * instance rmax: 128 or 512, one warp up to 128 (rmax 128 takes n <= 128) or
+ * 512 entries; 1024, and 512 above 512 entries, a team of warps:
  * order[k] = index of the entry at position k.  For checking it against
  * other implementations.  PIC_ERR_ARG on other n or rmax. */
 pic_status pic_order_check(const uint64_t *key, const uint64_t *id, int n, int rmax, uint16_t *order);

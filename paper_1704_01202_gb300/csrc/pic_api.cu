@@ -109,8 +109,6 @@ struct pic_ctx {
     int nsm = 0, grid_main = 0, grid_t1 = 0, grid_t2 = 0, grid_big = 0, grid_push = 0;
     NewE *nw = nullptr;                  // created-electron scratch of the cell launches
     size_t nw_entries = 0;
-    unsigned long long *gw = nullptr;    // global staging of the large-cell instances (ids, radix buffer)
-    size_t gw_words = 0;
     int64_t launches = 0;
     bool loaded_e = false, loaded_i = false;
     std::vector<double> hv_tab, sigma;   // host copy of the photoionization table
@@ -189,16 +187,6 @@ size_t nw_scratch_entries(int ncell)
     return warps * 768;
 }
 
-// Global staging of the large-cell instances, in 8-byte words: 3072 a warp
-// (ids, keys and positions of 1024 electrons in the FP32 build) for as many
-// warps; the
-// large cells' warps are few, and their grids are clamped to the slices.
-size_t gw_scratch_words(int ncell)
-{
-    const size_t warps = std::min<size_t>(192 * 16, (size_t)ncell + 64);
-    return warps * 3072;
-}
-
 size_t arena_need(int ncell, int npts, int nblk, int cap_e, int cap_i, int nslot, int nrows)
 {
     size_t b = 0;
@@ -211,7 +199,7 @@ size_t arena_need(int ncell, int npts, int nblk, int cap_e, int cap_i, int nslot
     b += 3 * al((size_t)npts * 3 * sizeof(real)) + al((size_t)npts * 3 * 8) + al((size_t)npts * 4);
     b += 2 * al((size_t)nrows * 4);
     b += al((size_t)ncell * PIC_MAX_BINS * sizeof(ph2));
-    b += al(nw_scratch_entries(ncell) * sizeof(NewE)) + al(gw_scratch_words(ncell) * 8);
+    b += al(nw_scratch_entries(ncell) * sizeof(NewE));
     b += al((4 + NZ + 4096 + 8) * 8);
     return b + 4096;
 }
@@ -234,20 +222,32 @@ double sigma_table(const pic_ctx *c, int s, double hv)
     return std::exp(std::log(v[lo]) + f * std::log(v[lo + 1] / v[lo]));
 }
 
-// the cell-kernel instance for a launch staging up to ce electrons and ci
-// ions per cell: in-register sorts up to 128, 512 or 1024 entries
+// Warps per cell of a launch staging up to ce electrons and ci ions: one
+// warp sorts up to 512 entries in registers; larger cells take a block of
+// TEAM warps, which share the staging (a 1024-electron cell's is ~50 KB: at
+// one warp a cell, 8 warps an SM): 700 cells of ~820 electrons and 102 ions,
+// 217 us a step at one warp a cell, 136 us at four.
+constexpr int TEAM = 4;
+int team_warps(int ce, int ci) { return std::max(ce, ci) > 512 ? TEAM : 1; }
+
+// the cell-kernel instance of such a launch
 typedef void (*CellKernel)(CellArgs);
 CellKernel cell_kernel(int ce, int ci)
 {
-    const int r = rmax_for(ce, ci);
-    return r == 128 ? k_cell<128> : (r == 512 ? k_cell<512> : k_cell<1024>);
+    if (team_warps(ce, ci) > 1) return k_cell<2048, TEAM>;
+    return std::max(ce, ci) <= 128 ? k_cell<128, 1> : k_cell<512, 1>;
 }
 
+// shared memory of a CTA of wpc warps (wpc / team_warps cells)
+size_t cell_smem(int ce, int ci, int wpc) { return cell_mem_bytes(ce, ci) * (wpc / team_warps(ce, ci)); }
+
 // largest warps per CTA of the cell kernel whose staging fits 200 KB, at
-// most 8 and at most what the instance's launch bounds allow
+// most 8 and at most what the instance's launch bounds allow; a team is a
+// CTA
 int max_wpc(int ce, int ci)
 {
-    const size_t per = warp_mem_bytes(ce, ci);
+    if (team_warps(ce, ci) > 1) return team_warps(ce, ci);
+    const size_t per = cell_mem_bytes(ce, ci);
     int lim = 8;
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, cell_kernel(ce, ci)) == cudaSuccess && fa.maxThreadsPerBlock >= 32)
@@ -256,12 +256,10 @@ int max_wpc(int ce, int ci)
 }
 
 // CTAs of a persistent cell launch staging ce / ci: the resident ones on
-// every SM, as many as the global scratches have warp slices for
+// every SM, as many as the global scratch has team slices for
 int cell_grid(const pic_ctx *c, int occ, int wpc, int ce, int ci)
 {
-    size_t cap = c->nw_entries / ((size_t)wpc * 3 * ci);
-    const size_t gw = warp_gmem_words(ce, ci);
-    if (gw) cap = std::min(cap, c->gw_words / ((size_t)wpc * gw));
+    const size_t cap = c->nw_entries / ((size_t)(wpc / team_warps(ce, ci)) * 3 * ci);
     return std::max(1, (int)std::min<size_t>((size_t)std::max(1, occ) * c->nsm, std::min<size_t>(cap, 1 << 30)));
 }
 
@@ -273,7 +271,7 @@ pic_status cell_smem_attr(pic_ctx *c)
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const size_t m = std::max(std::max(c->smem_main, c->smem_t1), std::max(c->smem_t2, c->smem_big));
-    for (CellKernel k : {k_cell<128>, k_cell<512>, k_cell<1024>}) {
+    for (CellKernel k : {k_cell<128, 1>, k_cell<512, 1>, k_cell<2048, TEAM>}) {
         cudaFuncAttributes fa{};
         CK(cudaFuncGetAttributes(&fa, k));
         const size_t lim = optin > (int)fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : m;
@@ -289,11 +287,12 @@ pic_status cell_smem_attr(pic_ctx *c)
 int best_wpc(pic_ctx *c, int ce, int ci)
 {
     if (cell_smem_attr(c) != PIC_OK) return max_wpc(ce, ci);
-    const size_t per = warp_mem_bytes(ce, ci);
+    if (team_warps(ce, ci) > 1) return team_warps(ce, ci);
     int best = 1, best_warps = 0;
     for (int w = 1; w <= max_wpc(ce, ci); ++w) {
         int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(ce, ci), 32 * w, per * w) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(ce, ci), 32 * w, cell_smem(ce, ci, w)) !=
+            cudaSuccess)
             continue;
         if (occ * w >= best_warps) { best_warps = occ * w; best = w; }
     }
@@ -304,7 +303,7 @@ int best_wpc(pic_ctx *c, int ce, int ci)
 pic_status set_wpc(pic_ctx *c, int wpc)
 {
     c->wpc = wpc;
-    c->smem_main = warp_mem_bytes(c->cap_ce, c->cap_ci) * wpc;
+    c->smem_main = cell_smem(c->cap_ce, c->cap_ci, wpc);
     pic_status r = cell_smem_attr(c);
     if (r != PIC_OK) return r;
     int occ = 0;
@@ -358,12 +357,12 @@ pic_status configure_cell_launch(pic_ctx *c, const int *hist_e, const int *hist_
         c->t1_ce = round_cap(want_e, 128, ce, 1024);
         c->t1_ci = round_cap(want_i, 32, ci, 256);
         c->t1_wpc = best_wpc(c, c->t1_ce, c->t1_ci);
-        c->smem_t1 = warp_mem_bytes(c->t1_ce, c->t1_ci) * c->t1_wpc;
+        c->smem_t1 = cell_smem(c->t1_ce, c->t1_ci, c->t1_wpc);
         if (want_e > c->t1_ce || want_i > c->t1_ci) {
             c->t2_ce = round_cap(want_e, 256, c->t1_ce, BIG_CE);
             c->t2_ci = round_cap(want_i, 64, c->t1_ci, BIG_CI);
             c->t2_wpc = best_wpc(c, c->t2_ce, c->t2_ci);
-            c->smem_t2 = warp_mem_bytes(c->t2_ce, c->t2_ci) * c->t2_wpc;
+            c->smem_t2 = cell_smem(c->t2_ce, c->t2_ci, c->t2_wpc);
         }
     }
     int wpc = best_wpc(c, ce, ci);
@@ -415,7 +414,6 @@ CellArgs cell_args(pic_ctx *c, CellTier tier)
     a.eos = c->d_eos;
     a.err = c->counters + CNT_ERR;
     a.nw = c->nw;
-    a.gw = c->gw;
     if (tier == TIER0) {
         a.work = c->counters + CNT_WORK;
         a.list = nullptr; a.n_list = nullptr;
@@ -590,7 +588,7 @@ pic_status launch_step(pic_ctx *c)
         ++c->launches;
     }
     CellArgs ab = cell_args(c, TIER_BIG);
-    cell_kernel(BIG_CE, BIG_CI)<<<c->grid_big, 32, c->smem_big, st>>>(ab);
+    cell_kernel(BIG_CE, BIG_CI)<<<c->grid_big, 32 * TEAM, c->smem_big, st>>>(ab);
     c->launches += 2;
     if (c->cell_ev_on) CK(cudaEventRecord(c->cell_ev[1], st));
     CK(cudaGetLastError());
@@ -834,8 +832,6 @@ pic_status ctx_create(pic_ctx **out, int nslot, int slot_cells, int slot_pts, in
     c->photons = carve_arena<ph2>(c, (size_t)c->ncell * PIC_MAX_BINS);
     c->nw_entries = nw_scratch_entries(c->ncell);
     c->nw = carve_arena<NewE>(c, c->nw_entries);
-    c->gw_words = gw_scratch_words(c->ncell);
-    c->gw = carve_arena<unsigned long long>(c, c->gw_words);
     c->diag_buf = carve_arena<double>(c, 4 + NZ + 4096 + 8);
     if (!c->diag_buf) { pic_free(c); return PIC_ERR_OOM; }
 
@@ -882,8 +878,8 @@ pic_status ctx_create(pic_ctx **out, int nslot, int slot_cells, int slot_pts, in
     } while (0);
     pic_status rc = PIC_OK;
     if (e != cudaSuccess) { rc = cuda_fail(c, e, "init copies"); pic_free(c); return rc; }
-    c->smem_big = warp_mem_bytes(BIG_CE, BIG_CI);
-    c->grid_big = cell_grid(c, 1, 1, BIG_CE, BIG_CI);
+    c->smem_big = cell_mem_bytes(BIG_CE, BIG_CI);
+    c->grid_big = cell_grid(c, 1, TEAM, BIG_CE, BIG_CI);
     e = cudaFuncSetAttribute(k_march, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * 8);
     if (e != cudaSuccess) { rc = cuda_fail(c, e, "march attribute"); pic_free(c); return rc; }
     {
@@ -1307,8 +1303,12 @@ pic_status tune_step(pic_ctx *c, int n, int &k)
         t = &c->tuned.back();
     }
     const int top = max_wpc(c->cap_ce, c->cap_ci);
-    int shapes = 0;
+    int shapes = 0, first = 0;
     while (shapes < 4 && (1 << shapes) <= top) ++shapes;
+    if (team_warps(c->cap_ce, c->cap_ci) > 1) {          // a team has one shape
+        first = 2;
+        shapes = 1;
+    }
     if (c->steps_done == 0 && k < n) {          // untimed first step of the context
         pic_status r = launch_step(c);
         if (r != PIC_OK) return r;
@@ -1321,7 +1321,7 @@ pic_status tune_step(pic_ctx *c, int n, int &k)
     }
     pic_status r = PIC_OK;
     while (t->tried < (unsigned)(2 * shapes) && k < n && r == PIC_OK) {
-        const int idx = t->tried < (unsigned)shapes ? (int)t->tried : 2 * shapes - 1 - (int)t->tried;
+        const int idx = first + (t->tried < (unsigned)shapes ? (int)t->tried : 2 * shapes - 1 - (int)t->tried);
         if ((r = set_wpc(c, 1 << idx)) != PIC_OK) break;
         c->cell_ev_on = true;
         r = launch_step(c);
@@ -1343,7 +1343,7 @@ pic_status tune_step(pic_ctx *c, int n, int &k)
     t->wpc = best_wpc(c, c->cap_ce, c->cap_ci);  // undecided: the default
     if (t->done) {
         float best = 3.4e38f;
-        for (int q = 0; q < shapes; ++q)
+        for (int q = first; q < first + shapes; ++q)
             if (t->ms[q] < best) { best = t->ms[q]; t->wpc = 1 << q; }
     }
     return set_wpc(c, t->wpc);
@@ -2023,9 +2023,14 @@ pic_status pic_order_check(const uint64_t *key, const uint64_t *id, int n, int r
     if (!key || !id || !order || n <= 0 || n > 4096 || !(rmax == 128 || rmax == 512 || rmax == 1024) ||
         (rmax == 128 && n > 128))
         return PIC_ERR_ARG;
-    const size_t smem = (size_t)n * 32 + 256 * 4 + (size_t)n * 2;
+    // one warp up to 128 or 512 entries, a team above (four warps, whose
+    // shares hold 2048; eight for the rest of the range)
+    const bool team = rmax == 1024 || n > 512;
+    const int warps = !team ? 1 : (n <= 512 * TEAM ? TEAM : 8);
+    const size_t smem = (size_t)n * 8;
     void (*kern)(const unsigned long long *, const unsigned long long *, int, unsigned short *) =
-        rmax == 128 ? k_order_check<128> : (rmax == 512 ? k_order_check<512> : k_order_check<1024>);
+        warps == 8 ? k_order_check<4096, 8> : warps == TEAM ? k_order_check<2048, TEAM>
+        : rmax == 128 ? k_order_check<128, 1> : k_order_check<512, 1>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return PIC_ERR_CUDA;
     char *d = nullptr;
@@ -2038,7 +2043,7 @@ pic_status pic_order_check(const uint64_t *key, const uint64_t *id, int n, int r
         cudaMemcpy(di, id, sizeof(uint64_t) * n, cudaMemcpyHostToDevice) != cudaSuccess)
         st = PIC_ERR_CUDA;
     if (st == PIC_OK) {
-        kern<<<1, 32, smem>>>(dk, di, n, dout);
+        kern<<<1, 32 * warps, smem>>>(dk, di, n, dout);
         if (cudaGetLastError() != cudaSuccess ||
             cudaMemcpy(order, dout, sizeof(uint16_t) * n, cudaMemcpyDeviceToHost) != cudaSuccess)
             st = PIC_ERR_CUDA;

@@ -1,11 +1,11 @@
-// Building blocks of the per-cell hot path: one warp owns one cell and runs,
-// in order, the canonical random ordering of its particles, the cell
-// moments (double-float sums), binary e-e and e-i collisions, Lotz impact
-// ionization, EOS-clamped recombination and, on rad steps, subshell
-// photoionization and K-vacancy decay (k_cell); the Boris push and the
-// charge-conserving deposit of the cell's particles follow in a second
-// kernel in the same canonical order (k_push).  Particles are staged in
-// shared memory; their positions stay in global memory until the push.
+// Building blocks of the per-cell hot path: one warp (or, for large cells, a
+// block of four) owns one cell and runs, in order, the canonical random
+// ordering of its particles, the cell moments (double-float sums), binary
+// e-e and e-i collisions, Lotz impact ionization, EOS-clamped recombination
+// and, on rad steps, subshell photoionization and K-vacancy decay (k_cell);
+// the Boris push and the charge-conserving deposit of the cell's particles
+// follow in a second kernel in the same canonical order (k_push).
+// Particles are staged in shared memory in that order.
 //
 // Determinism: every random number is keyed by (slab seed, particle id,
 // step, purpose) and every ordering comes from a sort on Philox keys, so
@@ -25,7 +25,7 @@ constexpr double JFIX = sizeof(real) == 8 ? 281474976710656.0 : 1099511627776.0;
 
 struct NewE {            // an electron created in this cell this step
     real ux, uy, uz, w;
-    int meta;            // ion slot | kind << 16
+    int meta;            // ion (position in the canonical order) | kind << 16
 };
 
 struct CellArgs {
@@ -58,8 +58,7 @@ struct CellArgs {
     const int *n_list;   // number of cells in the list (device)
     int *ovf_list, *ovf_count;   // cells too large for this pass
     int cap_ce, cap_ci, cap_new; // per-cell capacities (staging; created electrons)
-    NewE *nw;            // created-electron scratch: cap_new entries per warp of the launch
-    unsigned long long *gw;  // global staging: warp_gmem_words(cap_ce, cap_ci) words per warp
+    NewE *nw;            // created-electron scratch: cap_new entries per team of the launch
 };
 
 // warp reductions: a fixed tree, result broadcast from lane 0 so every lane
@@ -71,34 +70,62 @@ __device__ __forceinline__ real wsum_f(real v)
     return __shfl_sync(FULL, v, 0);
 }
 
+// dd_add is symmetric (TwoSum is exact either way round), so the butterfly
+// gives every lane the bits of the tree (lane l + lane l + 16, then + 8, ...)
 __device__ __forceinline__ dd wsum_dd(dd v)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        dd t{__shfl_down_sync(FULL, v.hi, o), __shfl_down_sync(FULL, v.lo, o)};
+        dd t{__shfl_xor_sync(FULL, v.hi, o), __shfl_xor_sync(FULL, v.lo, o)};
         v = dd_add(v, t);
-    }
-    return dd{__shfl_sync(FULL, v.hi, 0), __shfl_sync(FULL, v.lo, 0)};
-}
-
-__device__ __forceinline__ int wsum_i(int v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-    return __shfl_sync(FULL, v, 0);
-}
-
-// inclusive prefix over the lanes (fixed order)
-__device__ __forceinline__ real wscan_f(real v, int lane)
-{
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        real t = __shfl_up_sync(FULL, v, o);
-        if (lane >= o) v += t;
     }
     return v;
 }
 
+// Two or four sums at once over the same trees: each level halves the lanes
+// a sum needs, so the other sums use them (four sums cost six levels of
+// arithmetic instead of twenty).
+__device__ __forceinline__ dd wswap_add(dd a, dd b, bool up, int o)
+{
+    const dd mine = up ? b : a, give = up ? a : b;
+    dd t{__shfl_xor_sync(FULL, give.hi, o), __shfl_xor_sync(FULL, give.lo, o)};
+    return dd_add(mine, t);
+}
+
+__device__ __forceinline__ dd wtail_add(dd v, int from)
+{
+    for (int o = from; o > 0; o >>= 1) {
+        dd t{__shfl_xor_sync(FULL, v.hi, o), __shfl_xor_sync(FULL, v.lo, o)};
+        v = dd_add(v, t);
+    }
+    return v;
+}
+
+__device__ __forceinline__ dd wlane_dd(dd v, int src)
+{
+    return dd{__shfl_sync(FULL, v.hi, src), __shfl_sync(FULL, v.lo, src)};
+}
+
+__device__ __forceinline__ void wsum_dd2(dd &a, dd &b, int lane)
+{
+    const dd v = wtail_add(wswap_add(a, b, lane & 16, 16), 8);
+    a = wlane_dd(v, 0);
+    b = wlane_dd(v, 16);
+}
+
+__device__ __forceinline__ void wsum_dd4(dd &a, dd &b, dd &c, dd &d, int lane)
+{
+    const dd p = wswap_add(a, b, lane & 16, 16), q = wswap_add(c, d, lane & 16, 16);
+    const dd v = wtail_add(wswap_add(p, q, lane & 8, 8), 4);
+    a = wlane_dd(v, 0);
+    b = wlane_dd(v, 16);
+    c = wlane_dd(v, 8);
+    d = wlane_dd(v, 24);
+}
+
+__device__ __forceinline__ int wsum_i(int v) { return __reduce_add_sync(FULL, v); }
+
+// inclusive prefix over the lanes (fixed order)
 __device__ __forceinline__ dd wscan_dd(dd v, int lane)
 {
 #pragma unroll
@@ -109,220 +136,220 @@ __device__ __forceinline__ dd wscan_dd(dd v, int lane)
     return v;
 }
 
-__device__ __forceinline__ dd wbcast_dd(dd v, int src)
-{
-    return dd{__shfl_sync(FULL, v.hi, src), __shfl_sync(FULL, v.lo, src)};
-}
+// ---------------------------------------------------------------------
+// canonical order inside a cell: ascending (64-bit Philox key, id)
+// ---------------------------------------------------------------------
+// The sort moves 32-bit words: the key's top 32 - SB bits over the entry's
+// index (SB bits).  A compare-exchange is then one shuffle and one min or
+// max, against two shuffles and a 64-bit compare for (48 key bits | index)
+// words.  Entries whose words share all their key bits (probability
+// ~ n^2 2^SB / 2^33 per cell: 2e-4 for 128 entries of one warp, a quarter
+// for 1000 of a team) are put in (key, id) order afterwards, each run of
+// them by the thread that finds its start, so the result is the full
+// (key, id) order whatever SB is.
 
-// Sort of the cells larger than the register sorts take (n > radix_min of
-// the kernel instance): a stable LSD radix sort (four 8-bit digits) of the
-// keys' high 32 bits packed with the slot, then the rare runs of equal high
-// words reordered by (low word, id) by one lane.  buf holds 2 n packed
-// entries, hist 256 counters.
-__host__ __device__ constexpr int radix_min(int rmax) { return rmax > 512 ? rmax : 512; }
-
-// the cell-kernel instance (largest register sort) of a staging of ce
-// electrons and ci ions per cell
-__host__ __device__ constexpr int rmax_for(int ce, int ci)
-{
-    return ce <= 128 && ci <= 128 ? 128 : (ce <= 512 && ci <= 512 ? 512 : 1024);
-}
-
-template <class IdT>
-__device__ void warp_radix(const unsigned long long *key, IdT *id, unsigned short *slot, unsigned long long *tmp,
-                           unsigned long long *buf, int *hist, int n, int lane)
-{
-    unsigned long long *A = buf, *B = buf + n;
-    for (int k = lane; k < n; k += 32) A[k] = (key[k] & 0xffffffff00000000ull) | (unsigned long long)k;
-    for (int pass = 0; pass < 4; ++pass) {
-        const int shift = 32 + 8 * pass;
-        for (int b = lane; b < 256; b += 32) hist[b] = 0;
-        __syncwarp();
-        for (int k = lane; k < n; k += 32) atomicAdd(hist + (int)((A[k] >> shift) & 255u), 1);
-        __syncwarp();
-        // exclusive scan of the 256 counts: eight per lane, then across lanes
-        int c[8], run = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) { c[q] = hist[lane * 8 + q]; run += c[q]; }
-        int incl = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += t;
-        }
-        int off = incl - run;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) { hist[lane * 8 + q] = off; off += c[q]; }
-        __syncwarp();
-        // stable scatter, 32 entries at a time in order
-        for (int base = 0; base < n; base += 32) {
-            const int k = base + lane;
-            const bool act = k < n;
-            const unsigned long long v = act ? A[k] : 0ull;
-            const int d = act ? (int)((v >> shift) & 255u) : -1;
-            const unsigned peers = __match_any_sync(FULL, d);
-            const int at = act ? hist[d] + __popc(peers & ((1u << lane) - 1u)) : 0;
-            __syncwarp();
-            if (act) {
-                B[at] = v;
-                if (lane == __ffs(peers) - 1) hist[d] += __popc(peers);
-            }
-            __syncwarp();
-        }
-        unsigned long long *t = A; A = B; B = t;
+// keys and ids of a cell's records: Philox draws of the ids
+struct RecKeys {
+    const real4 *p1;         // second record words of the cell's first particle
+    bool elec;
+    unsigned long long seed;
+    unsigned step;
+    __device__ __forceinline__ unsigned long long id(int k) const
+    {
+        return elec ? rec_eid(p1[k]) : (unsigned long long)rec_iid(p1[k]);
     }
-    // equal high words (rare): order those runs by (low word, id)
-    bool tie = false;
-    for (int k = lane; k + 1 < n; k += 32) tie |= (A[k] >> 32) == (A[k + 1] >> 32);
-    if (__any_sync(FULL, tie) && lane == 0) {
-        for (int k = 1; k < n; ++k) {
-            unsigned long long v = A[k];
-            int j = k - 1;
-            while (j >= 0 && (A[j] >> 32) == (v >> 32)) {
-                const int sa = (int)(A[j] & 0xffffu), sb = (int)(v & 0xffffu);
-                const bool gt = key[sa] > key[sb] || (key[sa] == key[sb] && id[sa] > id[sb]);
-                if (!gt) break;
-                A[j + 1] = A[j];
+    __device__ __forceinline__ unsigned long long full(unsigned long long i) const
+    {
+        const U4 r = draw(seed, i, step, elec ? PU_PAIR_E : PU_PAIR_I);
+        return ((unsigned long long)r.x << 32) | r.y;
+    }
+    __device__ __forceinline__ unsigned long long key(int k) const { return full(id(k)); }
+    __device__ __forceinline__ unsigned top(int k) const
+    {
+        return draw(seed, id(k), step, elec ? PU_PAIR_E : PU_PAIR_I).x;
+    }
+};
+// given keys and ids (the check entry)
+struct GivenKeys {
+    const unsigned long long *k_, *id_;
+    __device__ __forceinline__ unsigned long long id(int k) const { return id_[k]; }
+    __device__ __forceinline__ unsigned long long key(int k) const { return k_[k]; }
+    __device__ __forceinline__ unsigned top(int k) const { return (unsigned)(k_[k] >> 32); }
+};
+
+// ascending bitonic sort of 32 E words of one warp, entry lane * E + j in
+// v[j]; rolled over the sizes above E so that its code stays small
+template <int E>
+__device__ __forceinline__ void sort_words(unsigned (&v)[E], int lane)
+{
+#pragma unroll
+    for (int size = 2; size <= E; size <<= 1) {
+#pragma unroll
+        for (int st = size >> 1; st > 0; st >>= 1) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                if (j & st) continue;
+                // the last in-lane size alternates its direction by lane
+                const bool asc = size < E ? (j & size) == 0 : (lane & 1) == 0;
+                const unsigned lo = min(v[j], v[j | st]), hi = max(v[j], v[j | st]);
+                v[j] = asc ? lo : hi;
+                v[j | st] = asc ? hi : lo;
+            }
+        }
+    }
+#pragma unroll 1
+    for (int ls = 2; ls <= 32; ls <<= 1) {           // size = ls * E
+        const bool asc = (lane & ls) == 0;           // ls = 32: always
+#pragma unroll 1
+        for (int lm = ls >> 1; lm > 0; lm >>= 1) {
+            const bool keep_min = ((lane & lm) == 0) == asc;
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                const unsigned o = __shfl_xor_sync(FULL, v[j], lm);
+                v[j] = keep_min ? min(o, v[j]) : max(o, v[j]);
+            }
+        }
+#pragma unroll
+        for (int st = E >> 1; st > 0; st >>= 1) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                if (j & st) continue;
+                const unsigned lo = min(v[j], v[j | st]), hi = max(v[j], v[j | st]);
+                v[j] = asc ? lo : hi;
+                v[j | st] = asc ? hi : lo;
+            }
+        }
+    }
+}
+
+// Runs of entries whose words share their key bits into (key, id) order:
+// insertion within the run by the thread (of nt) at its start.  Permuting
+// a run leaves its words' key bits in place, so the other threads' run
+// boundaries do not move.
+template <class Keys>
+__device__ __noinline__ void order_ties(Keys K, unsigned *w, int n, int sb, int t, int nt)
+{
+    const unsigned mask = (1u << sb) - 1u;
+    for (int k = t; k + 1 < n; k += nt) {
+        const unsigned p = w[k] >> sb;
+        if ((w[k + 1] >> sb) != p || (k > 0 && (w[k - 1] >> sb) == p)) continue;
+        for (int q = k + 1; q < n && (w[q] >> sb) == p; ++q) {
+            const unsigned x = w[q];
+            const unsigned long long kx = K.key((int)(x & mask)), ix = K.id((int)(x & mask));
+            int j = q - 1;
+            while (j >= k) {
+                const int y = (int)(w[j] & mask);
+                const unsigned long long ky = K.key(y);
+                if (!(ky > kx || (ky == kx && K.id(y) > ix))) break;
+                w[j + 1] = w[j];
                 --j;
             }
-            A[j + 1] = v;
-        }
-    }
-    __syncwarp();
-    for (int k = lane; k < n; k += 32) slot[k] = (unsigned short)(A[k] & 0xffffu);
-    __syncwarp();
-    for (int k = lane; k < n; k += 32) tmp[k] = (unsigned long long)id[slot[k]];
-    __syncwarp();
-    for (int k = lane; k < n; k += 32) id[k] = (IdT)tmp[k];
-    __syncwarp();
-}
-
-// Sort of up to 32 E entries in registers, E per lane (entry lane * E + j):
-// the bitonic network over (key high 48 bits | slot) words, compare-exchange
-// through warp shuffles across lanes and in place within a lane.  That is
-// the (key, id) order unless two keys share their high 48 bits (probability
-// ~n^2 / 2^49 per cell); such runs are then put in (key, id) order by one
-// lane.  slot[k] gets the slot at position k, id[] the ids in that order
-// (through tmp, n entries of scratch, which may be the key array).
-template <int E, int S>
-__device__ __forceinline__ void reg_cmpx_in_lane(unsigned long long (&v)[E], int lane, int size)
-{
-    if constexpr (S < E) {
-#pragma unroll
-        for (int j = 0; j < E; ++j) {
-            if ((j & S) != 0) continue;
-            const bool asc = ((lane * E + j) & size) == 0;
-            const unsigned long long a = v[j], b = v[j ^ S];
-            if ((a > b) == asc) { v[j] = b; v[j ^ S] = a; }
+            w[j + 1] = x;
         }
     }
 }
 
-// runs of equal high 48 key bits of a (high 48 bits, slot) order into
-// (key, id) order: insertion within each run, by one lane
-template <class IdT>
-__device__ void order_ties(const unsigned long long *key, const IdT *id, unsigned short *slot, int n)
+// one warp: w[k] = (key bits | index) of the entry at canonical position k
+// of n <= 32 E entries.  Out of line: one copy serves both species.
+template <int E, class Keys>
+__device__ __noinline__ void order_warp(Keys K, unsigned *w, int n, int lane)
 {
-    for (int k = 1; k < n; ++k) {
-        const int sb = slot[k];
-        const unsigned long long kb = key[sb];
-        int j = k - 1;
-        while (j >= 0) {
-            const int sa = slot[j];
-            const unsigned long long ka = key[sa];
-            if ((ka >> 16) != (kb >> 16)) break;
-            if (!(ka > kb || (ka == kb && id[sa] > id[sb]))) break;
-            slot[j + 1] = (unsigned short)sa;
-            --j;
-        }
-        slot[j + 1] = (unsigned short)sb;
-    }
-}
-
-template <int E, class IdT>
-__device__ __forceinline__ void warp_sort_reg(const unsigned long long *key, IdT *id, unsigned short *slot,
-                                              unsigned long long *tmp, int n, int lane)
-{
-    unsigned long long v[E];
+    constexpr int SB = E == 1 ? 5 : E == 2 ? 6 : E == 4 ? 7 : E == 8 ? 8 : 9;
+    constexpr unsigned mask = (1u << SB) - 1u;
+    unsigned v[E];
+    // padding sorts last: an entry's word equals it only as entry 32 E - 1,
+    // and then there is no padding
 #pragma unroll
     for (int j = 0; j < E; ++j) {
-        const int k = lane * E + j;
-        v[j] = k < n ? (key[k] & ~0xffffull) | (unsigned long long)k : ~0ull;
+        const int k = j * 32 + lane;
+        v[j] = k < n ? (K.top(k) & ~mask) | (unsigned)k : ~0u;
     }
-    for (int size = 2; size <= 32 * E; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride >= E) {
-                const int lm = stride / E;
-#pragma unroll
-                for (int j = 0; j < E; ++j) {
-                    const int e = lane * E + j;
-                    const unsigned long long o = __shfl_xor_sync(FULL, v[j], lm);
-                    const bool keep_min = ((e & stride) == 0) == ((e & size) == 0);
-                    v[j] = keep_min ? (o < v[j] ? o : v[j]) : (o > v[j] ? o : v[j]);
-                }
-            } else if (stride == 1) {
-                reg_cmpx_in_lane<E, 1>(v, lane, size);
-            } else if (stride == 2) {
-                reg_cmpx_in_lane<E, 2>(v, lane, size);
-            } else if (stride == 4) {
-                reg_cmpx_in_lane<E, 4>(v, lane, size);
-            } else if (stride == 8) {
-                reg_cmpx_in_lane<E, 8>(v, lane, size);
-            } else {
-                reg_cmpx_in_lane<E, 16>(v, lane, size);
-            }
-        }
-    }
-    // neighbours with equal high words (the padding never compares: its
-    // positions are >= n)
+    sort_words<E>(v, lane);
     bool tie = false;
 #pragma unroll
-    for (int j = 0; j + 1 < E; ++j)
-        tie |= lane * E + j + 1 < n && (v[j] >> 16) == (v[j + 1] >> 16);
-    const unsigned long long nx = __shfl_down_sync(FULL, v[0], 1);
-    tie |= lane < 31 && lane * E + E < n && (v[E - 1] >> 16) == (nx >> 16);
-#pragma unroll
     for (int j = 0; j < E; ++j) {
         const int k = lane * E + j;
-        if (k < n) slot[k] = (unsigned short)(v[j] & 0xffffu);
+        const unsigned nx = j + 1 < E ? v[j + 1 < E ? j + 1 : 0] : __shfl_down_sync(FULL, v[0], 1);
+        tie |= k + 1 < n && (v[j] >> SB) == (nx >> SB);
+        if (k < n) w[k] = v[j];
     }
     __syncwarp();
     if (__any_sync(FULL, tie)) {
-        if (lane == 0) order_ties<IdT>(key, id, slot, n);
+        order_ties(K, w, n, SB, lane, 32);
         __syncwarp();
     }
-    for (int k = lane; k < n; k += 32) tmp[k] = (unsigned long long)id[slot[k]];
-    __syncwarp();
-    for (int k = lane; k < n; k += 32) id[k] = (IdT)tmp[k];
-    __syncwarp();
 }
 
-// the larger register sorts out of line: their 16-32 key registers would
-// otherwise raise the register pressure of the whole cell kernel
-template <int E, class IdT>
-__device__ __noinline__ void warp_sort_reg_call(const unsigned long long *key, IdT *id, unsigned short *slot,
-                                                unsigned long long *tmp, int n, int lane)
+// A team of TW warps (the whole block): each warp sorts a share of 32 E
+// entries in registers, then every entry finds its place by its rank in the
+// other shares (binary searches in shared memory).  w: n words out; buf:
+// n words of scratch.
+constexpr int TEAM_SB = 12;              // up to 4096 entries
+template <int E, int TW, class Keys>
+__device__ __noinline__ void order_team(Keys K, unsigned *w, unsigned *buf, int n, int warp, int lane)
 {
-    warp_sort_reg<E, IdT>(key, id, slot, tmp, n, lane);
+    constexpr unsigned mask = (1u << TEAM_SB) - 1u;
+    unsigned v[E];
+    const int base = warp * 32 * E;
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        const int k = base + j * 32 + lane;
+        v[j] = k < n ? (K.top(k) & ~mask) | (unsigned)k : ~0u;
+    }
+    sort_words<E>(v, lane);
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        const int k = base + lane * E + j;
+        if (k < n) buf[k] = v[j];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        if (base + lane * E + j >= n) continue;
+        int rank = lane * E + j;
+        for (int o = 0; o < TW; ++o) {
+            if (o == warp) continue;
+            int lo = o * 32 * E, hi = min(n, lo + 32 * E);   // first word above v[j]
+            const int b = lo;
+            while (lo < hi) {
+                const int md = (lo + hi) >> 1;
+                if (buf[md] < v[j]) lo = md + 1; else hi = md;
+            }
+            rank += max(lo - b, 0);
+        }
+        w[rank] = v[j];
+    }
+    __syncthreads();
+    bool tie = false;
+    for (int k = warp * 32 + lane; k + 1 < n; k += 32 * TW) tie |= (w[k] >> TEAM_SB) == (w[k + 1] >> TEAM_SB);
+    if (__syncthreads_or(tie)) {
+        order_ties(K, w, n, TEAM_SB, warp * 32 + lane, 32 * TW);
+        __syncthreads();
+    }
 }
 
-// The in-cell canonical order, ascending (key, id): in registers up to
-// RMAX entries (128, 512 or 1024: the kernel instance), the radix sort
-// above radix_min(RMAX).  slot[] must hold 0..n-1 on entry; n is at most
-// RMAX when rbuf is NULL (the staging of a kernel instance without the
-// radix buffer never holds more).
-template <class IdT, int RMAX = 512>
-__device__ void warp_sort(unsigned long long *key, IdT *id, unsigned short *slot, unsigned long long *tmp,
-                          unsigned long long *rbuf, int *rhist, int n, int lane)
+// the canonical order of a cell of n entries by a team of TW warps: w[k] &
+// (return value) is the index of the entry at position k (buf: a team's
+// scratch, n words)
+template <int RMAX, int TW, class Keys>
+__device__ __forceinline__ unsigned order_cell(const Keys &K, unsigned *w, unsigned *buf, int n, int warp, int lane)
 {
-    if (n > radix_min(RMAX)) { warp_radix<IdT>(key, id, slot, tmp, rbuf, rhist, n, lane); return; }
-    if (n <= 32) warp_sort_reg<1, IdT>(key, id, slot, tmp, n, lane);
-    else if (n <= 64) warp_sort_reg<2, IdT>(key, id, slot, tmp, n, lane);
-    else if (n <= 128) warp_sort_reg<4, IdT>(key, id, slot, tmp, n, lane);
-    else if constexpr (RMAX > 128) {
-        if (n <= 256) warp_sort_reg_call<8, IdT>(key, id, slot, tmp, n, lane);
-        else if (n <= 512) warp_sort_reg_call<16, IdT>(key, id, slot, tmp, n, lane);
-        else if constexpr (RMAX > 512) warp_sort_reg_call<32, IdT>(key, id, slot, tmp, n, lane);
+    if constexpr (TW == 1) {
+        if (n <= 32) { order_warp<1>(K, w, n, lane); return 31u; }
+        if (n <= 64) { order_warp<2>(K, w, n, lane); return 63u; }
+        if (RMAX <= 128 || n <= 128) { order_warp<4>(K, w, n, lane); return 127u; }
+        if constexpr (RMAX > 128) {
+            if (n <= 256) { order_warp<8>(K, w, n, lane); return 255u; }
+            order_warp<16>(K, w, n, lane);
+        }
+        return 511u;
+    } else {
+        if (n <= 32 * TW) order_team<1, TW>(K, w, buf, n, warp, lane);
+        else if (n <= 64 * TW) order_team<2, TW>(K, w, buf, n, warp, lane);
+        else if (n <= 128 * TW) order_team<4, TW>(K, w, buf, n, warp, lane);
+        else if (n <= 256 * TW) order_team<8, TW>(K, w, buf, n, warp, lane);
+        else order_team<16, TW>(K, w, buf, n, warp, lane);
+        return (1u << TEAM_SB) - 1u;
     }
 }
 
@@ -332,105 +359,68 @@ __device__ __forceinline__ real cic_w(real x, int node)
     return d < RF(1.0) ? RF(1.0) - d : RF(0.0);
 }
 
-// per-warp shared memory carve-up
-struct WarpMem {
-    real4 *eu;                 // [cap_ce] ux uy uz w (slot order)
-    unsigned long long *ekey;   // [cap_ce] sort key, later reused as real take
-    unsigned long long *eid;    // [cap_ce] ids in canonical order
-    unsigned short *eperm;      // [cap_ce] canonical position -> slot
-    real2 *epos;               // [cap_ce] positions in the cell (slot order)
-    real2 *ipos;               // [cap_ci] ion positions in the cell (slot order)
-    real4 *iu;                 // [cap_ci] ux uy uz zfrac (slot order)
-    int *ist;                   // [cap_ci] Z | nK << 8 (slot order)
-    unsigned long long *ikey;   // [cap_ci] sort key, later reused as nrec
-    unsigned int *iid;          // [cap_ci] ids in canonical order
-    unsigned short *iperm;      // [cap_ci]
-    NewE *nw;                   // [cap_new] in global memory: the warp's slice of the scratch
+// Shared-memory staging of one cell, by the team (one warp, or the whole
+// block) that owns it.  Every array is in the cell's canonical order: a
+// warp's lanes read neighbouring entries, without bank conflicts and
+// without an index to load first.
+struct CellMem {
+    real4 *eu;                 // [cap_ce] ux uy uz w
+    real2 *epos;               // [cap_ce] positions in the cell
+    unsigned long long *eid;    // [cap_ce]
+    real2 *ew;                 // [max(cap_ce, cap_ci)] scratch: sort words; kinetic energy and w beta of each
+                                //   electron; weight taken by recombination
+    real4 *iu;                 // [cap_ci] ux uy uz zfrac
+    real2 *ipos;               // [cap_ci]
+    int *ist;                   // [cap_ci] Z | nK << 8
+    unsigned int *iid;          // [cap_ci]
+    int *nrec;                  // [cap_ci] recombinations of each ion
+    NewE *nw;                   // [cap_new] in global memory: the team's slice of the scratch
     real *dE;                  // [16] continuum lowering per charge state
     real *Pz;                  // [16] impact-ionization probability per charge
-    real4 *lz;                 // [NS] Lotz constants of one charge state: P, 1/P, ln P, a q
-    unsigned long long *rbuf;   // [2 max(cap_ce, cap_ci)] radix sort (only when a cell can exceed radix_min)
-    int *rhist;                 // [256]
+    real4 *lz;                 // [4][NS] Lotz constants of a charge state (one set per warp): P, 1/P, ln P, a q
     dd *ph;                     // [2 MAXB] photon bin scratch
     int *phc;                   // [MAXB] events per bin so far
+    dd *bc;                     // [8] sums a warp hands to its team
 };
 
-// shared-memory pieces start on 16 B (FP32) or 32 B (FP64: real4 is 32 B);
-// the sort-key storage later holds a real2 per electron
+// shared-memory pieces start on 16 B (FP32) or 32 B (FP64: real4 is 32 B)
 constexpr size_t kSmAlign = sizeof(real4) > 16 ? 32 : 16;
-constexpr size_t kKeyBytes = sizeof(real2) > 8 ? sizeof(real2) : 8;
 __host__ __device__ inline size_t amem(size_t x) { return (x + kSmAlign - 1) & ~(kSmAlign - 1); }
 
-// Shared memory of one warp staging up to ce electrons and ci ions.  The
+// Shared memory of a team staging up to ce electrons and ci ions.  The
 // electrons a cell creates in a step (up to 3 per ion: impact, photo- and
-// Auger ionization) are rare; they live in the warp's slice of a global
-// scratch, which keeps the staging of large cells small.  The instances
-// for cells above 128 entries, whose staging limits the warps resident on
-// an SM, also keep the electron ids (read once per collision), the sort
-// keys (later the per-electron scratch of the Lotz sums and of
-// recombination), the positions (read back once, at the write-back) and
-// the radix buffer there (warp_gmem_words 8-byte words a warp).
-__host__ __device__ inline bool ids_in_gmem(int ce, int ci) { return rmax_for(ce, ci) > 128; }
-
-__host__ __device__ inline size_t warp_gmem_words(int ce, int ci)
+// Auger ionization) are rare; they live in the team's slice of a global
+// scratch, which keeps the staging of large cells small.
+__host__ __device__ inline size_t cell_mem_bytes(int ce, int ci)
 {
-    if (!ids_in_gmem(ce, ci)) return 0;
     const int cm = ce > ci ? ce : ci;
-    return (size_t)ce * (1 + kKeyBytes / 8 + sizeof(real2) / 8) +
-           (cm > radix_min(rmax_for(ce, ci)) ? 2 * (size_t)cm : 0);
+    return amem((size_t)ce * sizeof(real4)) + amem((size_t)ce * sizeof(real2)) + amem((size_t)ce * 8) +
+           amem((size_t)cm * sizeof(real2)) + amem((size_t)ci * sizeof(real4)) + amem((size_t)ci * sizeof(real2)) +
+           3 * amem((size_t)ci * 4) + 2 * amem(16 * sizeof(real)) + amem(4 * NS * sizeof(real4)) +
+           amem(2 * MAXB * sizeof(dd)) + amem(MAXB * 4) + amem(8 * sizeof(dd));
 }
 
-__host__ __device__ inline size_t warp_mem_bytes(int ce, int ci)
+__device__ inline CellMem carve(char *base, int ce, int ci, NewE *nw)
 {
-    const bool g = ids_in_gmem(ce, ci);
-    size_t b = 0;
-    b += amem((size_t)ce * sizeof(real4)) +
-         (g ? 0 : amem((size_t)ce * kKeyBytes) + amem((size_t)ce * 8) + amem((size_t)ce * sizeof(real2))) +
-         amem((size_t)ce * 2) + amem((size_t)ci * sizeof(real2));
-    b += amem((size_t)ci * sizeof(real4)) + amem((size_t)ci * 4) + amem((size_t)ci * 8) + amem((size_t)ci * 4)
-         + amem((size_t)ci * 2);
-    b += amem(16 * sizeof(real)) * 2 + amem(NS * sizeof(real4)) + amem(2 * MAXB * sizeof(dd)) + amem(MAXB * 4);
+    CellMem m;
     const int cm = ce > ci ? ce : ci;
-    if (cm > radix_min(rmax_for(ce, ci))) b += (g ? 0 : amem((size_t)cm * 16)) + 256 * 4;
-    return b;
-}
-
-// gw: the warp's slice of the global staging (warp_gmem_words words)
-__device__ inline WarpMem carve(char *base, int ce, int ci, NewE *nw, unsigned long long *gw)
-{
-    const bool g = ids_in_gmem(ce, ci);
-    WarpMem m;
     char *p = base;
     m.eu = (real4 *)p; p += amem((size_t)ce * sizeof(real4));
-    if (g) {
-        m.eid = gw;
-        m.ekey = gw + ce;
-        m.epos = reinterpret_cast<real2 *>(gw + (size_t)ce * (1 + kKeyBytes / 8));
-    } else {
-        m.ekey = (unsigned long long *)p; p += amem((size_t)ce * kKeyBytes);
-        m.eid = (unsigned long long *)p; p += amem((size_t)ce * 8);
-        m.epos = (real2 *)p; p += amem((size_t)ce * sizeof(real2));
-    }
-    m.eperm = (unsigned short *)p; p += amem((size_t)ce * 2);
-    m.ipos = (real2 *)p; p += amem((size_t)ci * sizeof(real2));
+    m.epos = (real2 *)p; p += amem((size_t)ce * sizeof(real2));
+    m.eid = (unsigned long long *)p; p += amem((size_t)ce * 8);
+    m.ew = (real2 *)p; p += amem((size_t)cm * sizeof(real2));
     m.iu = (real4 *)p; p += amem((size_t)ci * sizeof(real4));
+    m.ipos = (real2 *)p; p += amem((size_t)ci * sizeof(real2));
     m.ist = (int *)p; p += amem((size_t)ci * 4);
-    m.ikey = (unsigned long long *)p; p += amem((size_t)ci * 8);
     m.iid = (unsigned int *)p; p += amem((size_t)ci * 4);
-    m.iperm = (unsigned short *)p; p += amem((size_t)ci * 2);
+    m.nrec = (int *)p; p += amem((size_t)ci * 4);
     m.nw = nw;
     m.dE = (real *)p; p += amem(16 * sizeof(real));
     m.Pz = (real *)p; p += amem(16 * sizeof(real));
-    m.lz = (real4 *)p; p += amem(NS * sizeof(real4));
+    m.lz = (real4 *)p; p += amem(4 * NS * sizeof(real4));
     m.ph = (dd *)p; p += amem(2 * MAXB * sizeof(dd));
     m.phc = (int *)p; p += amem(MAXB * 4);
-    const int cm = ce > ci ? ce : ci;
-    m.rbuf = nullptr; m.rhist = nullptr;
-    if (cm > radix_min(rmax_for(ce, ci))) {
-        if (g) m.rbuf = gw + (size_t)ce * (1 + kKeyBytes / 8 + sizeof(real2) / 8);
-        else { m.rbuf = (unsigned long long *)p; p += amem((size_t)cm * 16); }
-        m.rhist = (int *)p;
-    }
+    m.bc = (dd *)p;
     return m;
 }
 

@@ -1,6 +1,6 @@
-// The per-cell collision and atomic-process kernel k_cell: one warp per
-// cell, phase-synchronous rounds (see pic_cell.cuh for the building blocks;
-// the push and deposit follow in pic_push.cuh).
+// The per-cell collision and atomic-process kernel k_cell: one warp, or a
+// block of four, per cell (see pic_cell.cuh for the building blocks; the
+// push and deposit follow in pic_push.cuh).
 #pragma once
 #include <type_traits>
 #include "pic_cell.cuh"
@@ -16,8 +16,16 @@ struct WarpTally {
     int cnt[NCOUNT];
 };
 
-__device__ __forceinline__ void tally_flush(const CellArgs &a, WarpTally &w, int lane)
+// the counts every cell adds to, kept per lane and summed at the flush
+struct LaneTally { int ee, ei, ion, rej; };
+
+__device__ __forceinline__ void tally_flush(const CellArgs &a, WarpTally &w, LaneTally &l, int lane)
 {
+    w.cnt[C_EE] += wsum_i(l.ee);
+    w.cnt[C_EI] += wsum_i(l.ei);
+    w.cnt[C_ION] += wsum_i(l.ion);
+    w.cnt[C_ION_REJ] += wsum_i(l.rej);
+    l = LaneTally{0, 0, 0, 0};
     if (w.slab >= 0 && lane == 0) {
         SlabTally *tl = a.tally + w.slab;
         if (dd_f(w.ion) != RF(0.0)) atomicAdd(&tl->ion, (double)w.ion.hi + (double)w.ion.lo);
@@ -31,13 +39,12 @@ __device__ __forceinline__ void tally_flush(const CellArgs &a, WarpTally &w, int
     for (int q = 0; q < NCOUNT; ++q) w.cnt[q] = 0;
 }
 
-// per-cell scalars shared by the stages of one cell
+// per-cell scalars of the out-of-line stages
 struct CellCtx {
-    int s, lc, cx, cy, e0, ne, i0, ni;
-    unsigned step, flags;
+    int lc, ne, ni;
+    unsigned step;
     unsigned long long seed;
-    real wi, mi, n_e, n_i, nref;
-    bool rad;
+    real wi, n_i, nref;
     // sums the recombination stage needs, when the earlier stages already
     // hold them (every electron bulk, impact ionization run): kinetic
     // energy of the electrons after the ionization payment, their weight,
@@ -54,22 +61,27 @@ struct CellCtx {
 // draw); the mean momentum is shifted back to the cell's and the momenta
 // about it scaled by one factor (Newton) so that the cell's kinetic energy
 // is kept.  Sums are double-float (double-double in the FP64 build).
+__device__ __forceinline__ real gm1_free(real ux, real uy, real uz)
+{
+    return gm1_of(ux * ux + uy * uy + uz * uz);
+}
+
 struct ThermSums { dd W, K, Px, Py, Pz; int n; };
 
 __device__ __forceinline__ void therm_add(ThermSums &t, real4 u)
 {
     t.W = dd_addf(t.W, u.w);
-    t.K = dd_addf(t.K, u.w * (real)kMeC2 * gm1(u.x, u.y, u.z));
+    t.K = dd_addf(t.K, u.w * (real)kMeC2 * gm1_free(u.x, u.y, u.z));
     t.Px = dd_addf(t.Px, u.w * u.x); t.Py = dd_addf(t.Py, u.w * u.y); t.Pz = dd_addf(t.Pz, u.w * u.z);
     t.n += 1;
 }
 
-__device__ __noinline__ void stage_therm(const CellArgs &a, const WarpMem &m, const CellCtx &c, int lane, int nnew)
+__device__ __noinline__ void stage_therm(const CellMem &m, const CellCtx &c, int lane, int nnew)
 {
     const int ne = c.ne;
     const real MC2 = (real)kMeC2;
     ThermSums t0{dd_zero(), dd_zero(), dd_zero(), dd_zero(), dd_zero(), 0};
-    for (int k = lane; k < ne; k += 32) { real4 u = m.eu[m.eperm[k]]; if (u.w > RF(0.0)) therm_add(t0, u); }
+    for (int k = lane; k < ne; k += 32) { real4 u = m.eu[k]; if (u.w > RF(0.0)) therm_add(t0, u); }
     for (int k = lane; k < nnew; k += 32) {
         NewE q = m.nw[k];
         if (q.w > RF(0.0)) therm_add(t0, make_real4(q.ux, q.uy, q.uz, q.w));
@@ -90,18 +102,17 @@ __device__ __noinline__ void stage_therm(const CellArgs &a, const WarpMem &m, co
     };
     dd Qx = dd_zero(), Qy = dd_zero(), Qz = dd_zero();
     for (int k = lane; k < ne; k += 32) {
-        const int sl = m.eperm[k];
-        real4 u = m.eu[sl];
+        real4 u = m.eu[k];
         if (!(u.w > RF(0.0))) continue;
         real3 v = redraw(m.eid[k]);
-        m.eu[sl] = make_real4(v.x, v.y, v.z, u.w);
+        m.eu[k] = make_real4(v.x, v.y, v.z, u.w);
         Qx = dd_addf(Qx, u.w * v.x); Qy = dd_addf(Qy, u.w * v.y); Qz = dd_addf(Qz, u.w * v.z);
     }
     for (int k = lane; k < nnew; k += 32) {
         NewE q = m.nw[k];
         if (!(q.w > RF(0.0))) continue;
         const int islot = q.meta & 0xffff, kind = q.meta >> 16;
-        const unsigned ion_id = rec_iid(a.i1[c.i0 + islot]);
+        const unsigned ion_id = m.iid[islot];
         const unsigned long long id = ((unsigned long long)(((c.step + 1u) << 2) | (unsigned)kind) << 32) | ion_id;
         real3 v = redraw(id);
         q.ux = v.x; q.uy = v.y; q.uz = v.z;
@@ -118,10 +129,10 @@ __device__ __noinline__ void stage_therm(const CellArgs &a, const WarpMem &m, co
         auto one = [&](real4 u) {
             real dx = u.x - M[0], dy = u.y - M[1], dz = u.z - M[2];
             real ux = V[0] + s * dx, uy = V[1] + s * dy, uz = V[2] + s * dz;
-            e = dd_addf(e, u.w * MC2 * gm1(ux, uy, uz));
+            e = dd_addf(e, u.w * MC2 * gm1_free(ux, uy, uz));
             de = dd_addf(de, u.w * MC2 * (ux * dx + uy * dy + uz * dz) * r_rsqrt(RF(1.0) + ux * ux + uy * uy + uz * uz));
         };
-        for (int k = lane; k < ne; k += 32) { real4 u = m.eu[m.eperm[k]]; if (u.w > RF(0.0)) one(u); }
+        for (int k = lane; k < ne; k += 32) { real4 u = m.eu[k]; if (u.w > RF(0.0)) one(u); }
         for (int k = lane; k < nnew; k += 32) {
             NewE q = m.nw[k];
             if (q.w > RF(0.0)) one(make_real4(q.ux, q.uy, q.uz, q.w));
@@ -139,10 +150,9 @@ __device__ __noinline__ void stage_therm(const CellArgs &a, const WarpMem &m, co
         if (r_fabs(ds) <= RF(1e-7) * s) break;
     }
     for (int k = lane; k < ne; k += 32) {
-        const int sl = m.eperm[k];
-        real4 u = m.eu[sl];
+        real4 u = m.eu[k];
         if (!(u.w > RF(0.0))) continue;
-        m.eu[sl] = make_real4(V[0] + s * (u.x - M[0]), V[1] + s * (u.y - M[1]), V[2] + s * (u.z - M[2]), u.w);
+        m.eu[k] = make_real4(V[0] + s * (u.x - M[0]), V[1] + s * (u.y - M[1]), V[2] + s * (u.z - M[2]), u.w);
     }
     for (int k = lane; k < nnew; k += 32) {
         NewE q = m.nw[k];
@@ -154,8 +164,11 @@ __device__ __noinline__ void stage_therm(const CellArgs &a, const WarpMem &m, co
 }
 
 // ---- EOS-clamped three-body recombination (Sec. IV) ----
-__device__ __noinline__ void stage_recombine(const CellArgs &a, const WarpMem &m, const Tables &T, const SlabDev &S,
-                                             const CellCtx &c, int lane, real Wnew_imp, WarpTally &wt)
+// Run by one warp; a team's other warps join for the last pass, the
+// correction of every electron's energy (see recombine_apply).  Returns
+// whether events happened, with that pass's factor in delta.
+__device__ __noinline__ bool stage_recombine(const CellArgs &a, const CellMem &m, const Tables &T, const SlabDev &S,
+                                             const CellCtx &c, int lane, real Wnew_imp, WarpTally &wt, real &delta)
 {
     const int ne = c.ne, ni = c.ni;
     const real wi = c.wi, MC2 = (real)kMeC2;
@@ -169,12 +182,12 @@ __device__ __noinline__ void stage_recombine(const CellArgs &a, const WarpMem &m
         Wex = c.W_e;
     } else {
         real pq = RF(0.0);
-        for (int k = lane; k < ni; k += 32) { int sl = m.iperm[k]; pq += (real)(m.ist[sl] & 0xff) + m.iu[sl].w; }
+        for (int k = lane; k < ni; k += 32) pq += (real)(m.ist[k] & 0xff) + m.iu[k].w;
         zb = wsum_f(pq) / ni;
         dd pkb = dd_zero();
         real pwb = RF(0.0), pwx = RF(0.0);
         for (int k = lane; k < ne; k += 32) {
-            real4 u = m.eu[m.eperm[k]];
+            real4 u = m.eu[k];
             real ke = MC2 * gm1(u.x, u.y, u.z);
             pwx += u.w;
             if (S.E_bulk <= RF(0.0) || ke < S.E_bulk) { pwb += u.w; pkb = dd_addf(pkb, u.w * ke); }
@@ -186,14 +199,15 @@ __device__ __noinline__ void stage_recombine(const CellArgs &a, const WarpMem &m
     const real Te2 = Wb2 > RF(0.0) ? (RF(2.0) / RF(3.0)) * Kb2 / Wb2 : RF(0.0);
     const real zeos = eos_lookup(*a.eos, c.n_i, Te2);
     int Kev = zb > zeos ? (int)r_floor((zb - zeos) * ni + RF(0.5)) : 0;
+    if (Kev <= 0) return false;
     int pel = 0;
     for (int k = lane; k < ni; k += 32) pel += m.ist[k] & 0xff;
     const int elig = wsum_i(pel);
     Kev = min(Kev, elig);
     Kev = min(Kev, (int)r_floor(Wex / wi * (RF(1.0) + RF(1e-6))));
-    if (Kev <= 0) return;
-    int *nrec = (int *)m.ikey;            // sort keys are no longer needed
-    real *take = (real *)m.ekey;
+    if (Kev <= 0) return false;
+    int *nrec = m.nrec;
+    real *take = (real *)m.ew;
     for (int k = lane; k < ni; k += 32) nrec[k] = 0;
     __syncwarp();
     int left = Kev;
@@ -205,7 +219,7 @@ __device__ __noinline__ void stage_recombine(const CellArgs &a, const WarpMem &m
         for (int b0 = 0; b0 < ni && left > 0; b0 += 32) {
             int t = b0 + lane;
             bool e = false;
-            if (t < ni) e = (m.ist[m.iperm[t]] & 0xff) - nrec[t] >= 1;
+            if (t < ni) e = (m.ist[t] & 0xff) - nrec[t] >= 1;
             unsigned bal = __ballot_sync(FULL, e);
             int rank = __popc(bal & ((1u << lane) - 1u));
             if (e && rank < left) nrec[t] += 1;
@@ -213,61 +227,72 @@ __device__ __noinline__ void stage_recombine(const CellArgs &a, const WarpMem &m
             __syncwarp();
         }
     }
+    // the electron weight removed, in canonical order: once the weight
+    // passed is beyond it by more than rounding, the rest give nothing
+    // (weights are not negative)
     const dd Wrem = dd{(real)Kev * wi, RF(0.0)};
     dd carry = dd_zero(), remKE = dd_zero();
+    bool more = true;
     for (int b0 = 0; b0 < ne; b0 += 32) {
         int t = b0 + lane;
+        if (!more) {
+            if (t < ne) take[t] = RF(0.0);
+            continue;
+        }
         real w = RF(0.0), ke = RF(0.0);
-        if (t < ne) { real4 u = m.eu[m.eperm[t]]; w = u.w; ke = MC2 * gm1(u.x, u.y, u.z); }
+        if (t < ne) { real4 u = m.eu[t]; w = u.w; ke = MC2 * gm1(u.x, u.y, u.z); }
         dd incl = dd_add(carry, wscan_dd(dd{w, RF(0.0)}, lane));
         dd before = dd_sub(incl, dd{w, RF(0.0)});
         real tk = r_fmin(r_fmax(dd_f(dd_sub(Wrem, before)), RF(0.0)), w);
         if (t < ne) take[t] = tk;
         remKE = dd_addf(remKE, tk * ke);
-        carry = wbcast_dd(incl, 31);
+        carry = wlane_dd(incl, 31);
+        more = !(dd_f(dd_sub(Wrem, carry)) < -RF(1e-6) * Wrem.hi);
     }
     __syncwarp();
     remKE = wsum_dd(remKE);
     dd pb = dd_zero();
     for (int k = lane; k < ni; k += 32) {
-        int st = m.ist[m.iperm[k]];
+        int st = m.ist[k];
         int Z = st & 0xff, nK = (st >> 8) & 0xff;
         for (int r = 1; r <= nrec[k]; ++r) pb = dd_addf(pb, wi * removal_energy(T, Z - r, nK, m.dE[Z - r]));
     }
     const dd bind = wsum_dd(pb);
     dd pkr = dd_zero();
     for (int k = lane; k < ne; k += 32) {
-        real4 u = m.eu[m.eperm[k]];
+        real4 u = m.eu[k];
         real ke = MC2 * gm1(u.x, u.y, u.z);
         if (S.E_bulk <= RF(0.0) || ke < S.E_bulk) pkr = dd_addf(pkr, (u.w - take[k]) * ke);
     }
     const real Krem = dd_f(wsum_dd(pkr));
-    if (Krem > RF(0.0)) {
-        real delta = -dd_f(dd_add(remKE, bind)) / Krem;
-        for (int k = lane; k < ne; k += 32) {
-            int sl = m.eperm[k];
-            real4 u = m.eu[sl];
-            real ke = MC2 * gm1(u.x, u.y, u.z);
-            bool bulk = S.E_bulk <= RF(0.0) || ke < S.E_bulk;
-            real tk = take[k];
-            real wn = u.w - tk;
-            bool dead = tk > RF(0.0) && wn <= RF(0.0);
-            u.w = dead ? RF(0.0) : wn;
-            if (bulk && !dead) scale_kinetic(u.x, u.y, u.z, delta);
-            m.eu[sl] = u;
-        }
-        for (int k = lane; k < ni; k += 32) {
-            int sl = m.iperm[k];
-            m.ist[sl] = m.ist[sl] - nrec[k];
-        }
-        wt.ion = dd_sub(wt.ion, bind);
-        if (lane == 0) wt.cnt[C_REC] += Kev;
-    }
+    if (!(Krem > RF(0.0))) return false;
+    delta = -dd_f(dd_add(remKE, bind)) / Krem;
+    for (int k = lane; k < ni; k += 32) m.ist[k] = m.ist[k] - nrec[k];
+    wt.ion = dd_sub(wt.ion, bind);
+    wt.cnt[C_REC] += Kev;
     __syncwarp();
+    return true;
+}
+
+__device__ __forceinline__ void recombine_apply(const CellMem &m, const SlabDev &S, int ne, real delta, int t, int nt)
+{
+    const real *take = (const real *)m.ew;
+    const real E_bulk = S.E_bulk;
+    for (int k = t; k < ne; k += nt) {
+        real4 u = m.eu[k];
+        real ke = (real)kMeC2 * gm1(u.x, u.y, u.z);
+        bool bulk = E_bulk <= RF(0.0) || ke < E_bulk;
+        real tk = take[k];
+        real wn = u.w - tk;
+        bool dead = tk > RF(0.0) && wn <= RF(0.0);
+        u.w = dead ? RF(0.0) : wn;
+        if (bulk && !dead) scale_kinetic(u.x, u.y, u.z, delta);
+        m.eu[k] = u;
+    }
 }
 
 // ---- rad step: subshell photoionization (Eq. 2) ----
-__device__ __noinline__ void stage_photo(const CellArgs &a, const WarpMem &m, const Tables &T, const SlabDev &S,
+__device__ __noinline__ void stage_photo(const CellArgs &a, const CellMem &m, const Tables &T, const SlabDev &S,
                                          const CellCtx &c, int lane, int &nnew, WarpTally &wt)
 {
     const int ni = c.ni, nb = S.nb;
@@ -292,7 +317,7 @@ __device__ __noinline__ void stage_photo(const CellArgs &a, const WarpMem &m, co
         int sub = -1, bin = -1, sl = 0, Z = 0, nK = 0;
         real edge = RF(0.), rc = RF(0.), rp = RF(0.);
         if (t < ni) {
-            sl = m.iperm[t];
+            sl = t;
             int st = m.ist[sl];
             Z = st & 0xff; nK = (st >> 8) & 0xff;
             int occ[NS];
@@ -404,7 +429,7 @@ __device__ __noinline__ void stage_photo(const CellArgs &a, const WarpMem &m, co
 }
 
 // ---- rad step: K-vacancy decay with KLL Auger / K-alpha branching ----
-__device__ __noinline__ void stage_decay(const CellArgs &a, const WarpMem &m, const Tables &T, const SlabDev &S,
+__device__ __noinline__ void stage_decay(const CellArgs &a, const CellMem &m, const Tables &T, const SlabDev &S,
                                          const CellCtx &c, int lane, int &nnew, WarpTally &wt)
 {
     const int ni = c.ni, nb = S.nb;
@@ -419,7 +444,7 @@ __device__ __noinline__ void stage_decay(const CellArgs &a, const WarpMem &m, co
         int kind = 0, sl = 0, Z = 0;
         real EA = RF(0.), rc = RF(0.), rp = RF(0.), Eka = RF(0.);
         if (t < ni) {
-            sl = m.iperm[t];
+            sl = t;
             int st = m.ist[sl];
             Z = st & 0xff;
             int nK = (st >> 8) & 0xff;
@@ -489,27 +514,43 @@ __device__ __noinline__ void stage_decay(const CellArgs &a, const WarpMem &m, co
     __syncwarp();
 }
 
-// One round: every warp of the block takes at most one cell; the stages
-// are separated by block barriers so the warps of an SM fetch the same code
+// One cell by its team of TW warps (t of nt = 32 TW threads).  TW = 1: every
+// warp of the block takes at most one cell a round, and the stages are
+// separated by block barriers so that the warps of an SM fetch the same code
 // at the same time (the stages are long and the instruction cache small).
-template <int RMAX>
-__device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables &T, int g, int lane, WarpTally &wt)
+// TW > 1: the block owns one cell.  Per-particle work is spread over the
+// team; every sum is formed by one warp over the canonical order (lane-
+// strided, fixed tree), so it has the same bits whatever TW is.
+template <int TW>
+__device__ __forceinline__ void team_sync()
 {
+    if constexpr (TW == 1) __syncwarp();
+    else __syncthreads();
+}
+
+template <int RMAX, int TW>
+__device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &T, int g, int warp, int lane,
+                             WarpTally &wt, LaneTally &lt)
+{
+    constexpr int nt = 32 * TW;
+    const int t0 = TW == 1 ? lane : warp * 32 + lane;
+    // the warps of a team that form its sums (one warp: all of them)
+    const bool w0 = TW == 1 || warp == 0, w1 = TW == 1 || warp == 1, w2 = TW == 1 || warp == 2,
+               w3 = TW == 1 || warp == 3;
     bool on = g >= 0;
     int s = 0;
     const SlabDev *Sp = a.slabs;
     unsigned step = 0, flags = 0;
     unsigned long long seed = 0;
-    int lc = 0, cx = 0, cy = 0, e0 = 0, ne = 0, i0 = 0, ni = 0;
+    int lc = 0, e0 = 0, ne = 0, i0 = 0, ni = 0;
     if (on) {
         s = __ldg(a.cell_slab + g);
-        if (s != wt.slab) { tally_flush(a, wt, lane); wt.slab = s; }
+        if (s != wt.slab) { tally_flush(a, wt, lt, lane); wt.slab = s; }
         Sp = a.slabs + s;
         step = a.steps[s];
         seed = Sp->seed;
         flags = Sp->flags;
         lc = g - Sp->cell0;
-        cx = lc % Sp->nx; cy = lc / Sp->nx;
         e0 = a.cs_e[g]; ne = a.cs_e[g + 1] - e0;
         i0 = a.cs_i[g]; ni = a.cs_i[g + 1] - i0;
         on = (ne > 0 || ni > 0) && Sp->active;
@@ -517,13 +558,15 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
     const SlabDev &S = *Sp;
     const real wi = S.w_ion;
     const real mi = S.m_ion;
+    const real dt = S.dt;
     const bool rad = S.rad_every > 0 && (step % (unsigned)S.rad_every) == 0;
     const real MC2 = (real)kMeC2;
+    const real mw_i = r_mul(r_mul(wi, MC2), mi);      // kinetic energy of an ion per gamma - 1
     const real nref = S.nref_f;
-    int c_ee = 0, c_ei = 0, c_ion = 0, c_rej = 0;
     real n_e = RF(0.), n_i = RF(0.), Te = RF(0.), zbar = RF(0.), lnL = RF(2.);
     const bool coll = (flags & 3u) != 0;
-    const bool all_bulk = S.E_bulk <= RF(0.0);
+    const real E_bulk = S.E_bulk;
+    const bool all_bulk = E_bulk <= RF(0.0);
     dd Kpre = dd_zero();
     int nnew = 0;
     real Wnew_imp = RF(0.0);
@@ -534,159 +577,228 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
     bool ew_ready = false, ionized = false;
 
     if (on) {
-    // ---- stage in shared memory; Philox sort keys ----
-    for (int k = lane; k < ne; k += 32) {
-        real4 P0 = a.e0[e0 + k], P1 = a.e1[e0 + k];
-        m.eu[k] = make_real4(P0.z, P0.w, P1.x, P1.y);
-        m.epos[k] = make_real2(P0.x, P0.y);
-        unsigned long long id = rec_eid(P1);
-        U4 r = draw(seed, id, step, PU_PAIR_E);
-        m.ekey[k] = ((unsigned long long)r.x << 32) | r.y;
-        m.eid[k] = id;
-        m.eperm[k] = (unsigned short)k;
+    // ---- canonical order, then the records staged in it ----
+    unsigned *words = reinterpret_cast<unsigned *>(m.ew);
+    {
+        const RecKeys K{a.e1 + e0, true, seed, step};
+        for (int k = t0; k < ne; k += nt) prefetch_l2(a.e0 + e0 + k);
+        const unsigned mask = order_cell<RMAX, TW>(K, words, words + ne, ne, warp, lane);
+        for (int k = t0; k < ne; k += nt) {
+            const int sl = (int)(words[k] & mask);
+            const real4 P0 = a.e0[e0 + sl], P1 = a.e1[e0 + sl];
+            m.eu[k] = make_real4(P0.z, P0.w, P1.x, P1.y);
+            m.epos[k] = make_real2(P0.x, P0.y);
+            m.eid[k] = rec_eid(P1);
+        }
+        team_sync<TW>();
     }
-    for (int k = lane; k < ni; k += 32) {
-        real4 P0 = a.i0[i0 + k], P1 = a.i1[i0 + k];
-        m.iu[k] = make_real4(P0.z, P0.w, P1.x, P1.y);
-        m.ipos[k] = make_real2(P0.x, P0.y);
-        m.ist[k] = rec_ist(P1);
-        unsigned id = rec_iid(P1);
-        U4 r = draw(seed, (unsigned long long)id, step, PU_PAIR_I);
-        m.ikey[k] = ((unsigned long long)r.x << 32) | r.y;
-        m.iid[k] = id;
-        m.iperm[k] = (unsigned short)k;
+    {
+        const RecKeys K{a.i1 + i0, false, seed, step};
+        const unsigned mask = order_cell<RMAX, TW>(K, words, words + ni, ni, warp, lane);
+        for (int k = t0; k < ni; k += nt) {
+            const int sl = (int)(words[k] & mask);
+            const real4 P0 = a.i0[i0 + sl], P1 = a.i1[i0 + sl];
+            m.iu[k] = make_real4(P0.z, P0.w, P1.x, P1.y);
+            m.ipos[k] = make_real2(P0.x, P0.y);
+            m.ist[k] = rec_ist(P1);
+            m.iid[k] = rec_iid(P1);
+        }
+        team_sync<TW>();
     }
-    __syncwarp();
-    // the sorted keys are not needed after the sort: they serve as scratch
-    warp_sort<unsigned long long, RMAX>(m.ekey, m.eid, m.eperm, m.ekey, m.rbuf, m.rhist, ne, lane);
-    warp_sort<unsigned int, RMAX>(m.ikey, m.iid, m.iperm, m.ikey, m.rbuf, m.rhist, ni, lane);
-
     }
-    __syncthreads();
+    if constexpr (TW == 1) __syncthreads();
 
     if (on && rad && S.rt) {
     // ---- transport mode: the energy the radiation field gave up to (or
     //      took from) this cell goes to its bulk electrons by one factor on
     //      their kinetic energy (Sec. II), at most 90 % of it taken; the rest
     //      waits for the next rad step ----
+    if (w0) {
     if (lane < S.nb) S.rt_chi[(size_t)lc * S.nb + lane] = 0.0f;
     if (lane == 0) S.rt_emc[lc] = 0.0;
     const double dEc = S.rt_dE[lc];
     if (dEc != 0.0) {
         dd pk = dd_zero();
         for (int k = lane; k < ne; k += 32) {
-            const real4 u = m.eu[m.eperm[k]];
+            const real4 u = m.eu[k];
             const real ke = MC2 * gm1(u.x, u.y, u.z);
-            if (S.E_bulk <= RF(0.0) || ke < S.E_bulk) pk = dd_addf(pk, u.w * ke);
+            if (E_bulk <= RF(0.0) || ke < E_bulk) pk = dd_addf(pk, u.w * ke);
         }
         const real K = dd_f(wsum_dd(pk));
         if (K > RF(0.0)) {
             const real dEa = (real)dEc < -RF(0.9) * K ? -RF(0.9) * K : (real)dEc;
             const real delta = -dEa / K;
             for (int k = lane; k < ne; k += 32) {
-                const int sl = m.eperm[k];
-                real4 u = m.eu[sl];
+                real4 u = m.eu[k];
                 const real ke = MC2 * gm1(u.x, u.y, u.z);
-                if (S.E_bulk <= RF(0.0) || ke < S.E_bulk) { scale_kinetic(u.x, u.y, u.z, delta); m.eu[sl] = u; }
+                if (E_bulk <= RF(0.0) || ke < E_bulk) { scale_kinetic(u.x, u.y, u.z, delta); m.eu[k] = u; }
             }
             if (lane == 0) S.rt_dE[lc] = dEc - (double)dEa;
             wt.rt = dd_addf(wt.rt, dEa);
         }
     }
-    __syncwarp();
+    }
+    team_sync<TW>();
     }
 
     if (on) {
     // ---- cell moments (Sec. II: T_e = 2/3 E_ave over bulk electrons) ----
-    dd We = dd_zero(), Wb = dd_zero(), Kb = dd_zero(), Q = dd_zero(), Ka = dd_zero();
-    for (int k = lane; k < ne; k += 32) {
-        real4 u = m.eu[m.eperm[k]];
-        const real g1 = gm1(u.x, u.y, u.z);
-        const real ke = MC2 * g1;
-        // w * MC2 * g1: the same rounding as the kernel's other kinetic-energy
-        // sums, so that the collision energy restore does not see a bias
-        // between two formulas of the same energy
-        const real wk = u.w * MC2 * g1;
-        We = dd_addf(We, u.w);
-        if (all_bulk || ke < S.E_bulk) { Wb = dd_addf(Wb, u.w); Kb = dd_addf(Kb, wk); }
-        if (!all_bulk) Ka = dd_addf(Ka, wk);
+    // with every electron bulk (the default) the bulk sums are the sums
+    dd We = dd_zero(), Wb = dd_zero(), Kb = dd_zero(), Q = dd_zero(), Ka = dd_zero(), Ki = dd_zero();
+    if (all_bulk) {
+        if constexpr (TW == 1) {
+            for (int k = lane; k < ne; k += 32) {
+                const real4 u = m.eu[k];
+                const real g1 = gm1(u.x, u.y, u.z);
+                We = dd_addf(We, u.w);
+                Kb = dd_addf(Kb, r_mul(r_mul(u.w, MC2), g1));
+            }
+        } else {
+            if (w0) for (int k = lane; k < ne; k += 32) We = dd_addf(We, m.eu[k].w);
+            if (w1)
+                for (int k = lane; k < ne; k += 32) {
+                    const real4 u = m.eu[k];
+                    const real g1 = gm1(u.x, u.y, u.z);
+                    Kb = dd_addf(Kb, r_mul(r_mul(u.w, MC2), g1));
+                }
+        }
+    } else if (w0) {
+        for (int k = lane; k < ne; k += 32) {
+            const real4 u = m.eu[k];
+            const real g1 = gm1(u.x, u.y, u.z);
+            const real ke = MC2 * g1;
+            const real wk = r_mul(r_mul(u.w, MC2), g1);
+            We = dd_addf(We, u.w);
+            if (ke < E_bulk) { Wb = dd_addf(Wb, u.w); Kb = dd_addf(Kb, wk); }
+            Ka = dd_addf(Ka, wk);
+        }
     }
-    for (int k = lane; k < ni; k += 32) {
-        int sl = m.iperm[k];
-        Q = dd_addf(Q, (real)(m.ist[sl] & 0xff) + m.iu[sl].w);
+    if (w2) for (int k = lane; k < ni; k += 32) Q = dd_addf(Q, (real)(m.ist[k] & 0xff) + m.iu[k].w);
+    if (w3 && coll)
+        for (int k = lane; k < ni; k += 32) { real4 u = m.iu[k]; Ki = dd_addp(Ki, mw_i, gm1(u.x, u.y, u.z)); }
+    if constexpr (TW == 1) {
+        wsum_dd4(We, Kb, Q, Ki, lane);
+        if (!all_bulk) wsum_dd2(Wb, Ka, lane);
+    } else {
+        if (w0) {
+            We = wsum_dd(We);
+            if (lane == 0) m.bc[0] = We;
+            if (!all_bulk) {
+                Kb = wsum_dd(Kb); Wb = wsum_dd(Wb); Ka = wsum_dd(Ka);
+                if (lane == 0) { m.bc[1] = Kb; m.bc[4] = Wb; m.bc[5] = Ka; }
+            }
+        }
+        if (w1 && all_bulk) { Kb = wsum_dd(Kb); if (lane == 0) m.bc[1] = Kb; }
+        if (w2) { Q = wsum_dd(Q); if (lane == 0) m.bc[2] = Q; }
+        if (w3) { Ki = wsum_dd(Ki); if (lane == 0) m.bc[3] = Ki; }
+        __syncthreads();
+        We = m.bc[0]; Kb = m.bc[1]; Q = m.bc[2]; Ki = m.bc[3];
+        if (!all_bulk) { Wb = m.bc[4]; Ka = m.bc[5]; }
     }
-    We = wsum_dd(We); Wb = wsum_dd(Wb); Kb = wsum_dd(Kb); Q = wsum_dd(Q);
-    Kall = all_bulk ? Kb : wsum_dd(Ka);
+    if (all_bulk) { Wb = We; Ka = Kb; }
+    Kall = Ka;
     Qcell = Q;
     We_cell = dd_f(We);
     n_e = dd_f(We) * nref; n_i = (real)ni * wi * nref;
     Te = dd_f(Wb) > RF(0.0) ? (RF(2.0) / RF(3.0)) * dd_f(Kb) / dd_f(Wb) : RF(0.0);
     zbar = ni > 0 ? dd_f(Q) / ni : RF(0.0);
-    if (lane < NZ) m.dE[lane] = ipd_shift(S.ipd, lane, n_e, n_i, Te, zbar);
+    if (w0 && lane < NZ) m.dE[lane] = ipd_shift(S.ipd, lane, n_e, n_i, Te, zbar);
     lnL = S.coulomb_log > RF(0.0) ? S.coulomb_log : coulomb_log(n_e, Te, zbar);
-    __syncwarp();
+    if constexpr (TW == 1) __syncwarp();
 
     // ---- binary collisions (Sec. IV): e-e, then e-i; exact energy restore ----
-    if (coll) {
-        // electron part from the moments above; the ions' own pass
-        dd pki = dd_zero();
-        for (int k = lane; k < ni; k += 32) { real4 u = m.iu[m.iperm[k]]; pki = dd_addf(pki, wi * MC2 * mi * gm1(u.x, u.y, u.z)); }
-        Kpre = dd_add(Kall, wsum_dd(pki));
-    }
+    if (coll) Kpre = dd_add(Kall, Ki);
     if ((flags & 1u) && ne >= 2) {
-        const int start = (ne & 1) ? 3 : 0;
         auto ee = [&](int pa, int pb, real dtc) {
-            int sa = m.eperm[pa], sb = m.eperm[pb];
-            real4 A = m.eu[sa], B = m.eu[sb];
-            real3 ua = make_real3(A.x, A.y, A.z), ub = make_real3(B.x, B.y, B.z);
-            U4 r = draw(seed, m.eid[pa], step, PU_COLL_EE);
-            if (binary_collision(ua, ub, RF(1.0), RF(1.0), -RF(1.0), -RF(1.0), A.w, B.w, n_e, lnL, dtc,
-                                 u01(r.x), u01(r.y), u01(r.z), u01(r.w))) c_ee++;
-            m.eu[sa] = make_real4(ua.x, ua.y, ua.z, A.w);
-            m.eu[sb] = make_real4(ub.x, ub.y, ub.z, B.w);
+            const real4 A = m.eu[pa], B = m.eu[pb];
+            const U4 r = draw(seed, m.eid[pa], step, PU_COLL_EE);
+            const Collided q = binary_collision(A, B, RF(1.0), RF(1.0), -RF(1.0), -RF(1.0), A.w, B.w, n_e, lnL, dtc, r);
+            lt.ee += q.hit;
+            m.eu[pa] = q.a;
+            m.eu[pb] = q.b;
         };
-        if ((ne & 1) && lane == 0) {
-            ee(0, 1, RF(0.5) * S.dt);
-            ee(1, 2, RF(0.5) * S.dt);
-            ee(2, 0, RF(0.5) * S.dt);
-        }
+        // an odd count pairs its first three in a triangle at half the step
+        const int start = (ne & 1) ? 3 : 0;
         const int npairs = (ne - start) >> 1;
-        for (int p = lane; p < npairs; p += 32) ee(start + 2 * p, start + 2 * p + 1, S.dt);
-        __syncwarp();
+        if (start && t0 == 0)
+#pragma unroll 1
+            for (int q = 0; q < 3; ++q) ee(q, q == 2 ? 0 : q + 1, RF(0.5) * dt);
+#pragma unroll 1
+        for (int p = t0; p < npairs; p += nt) ee(start + 2 * p, start + 2 * p + 1, dt);
     }
-
+    team_sync<TW>();
     }
-    __syncthreads();     // the e-i code next: warps in step, as elsewhere
+    if constexpr (TW == 1) __syncthreads();     // the e-i code next: warps in step, as elsewhere
 
     if (on) {
     if ((flags & 2u) && ne >= 1 && ni >= 1) {
-        const bool e_long = ne >= ni;
-        const int nlong = e_long ? ne : ni, nshort = e_long ? ni : ne;
-        for (int base = 0; base < nlong; base += nshort) {
-            int cnt = min(nshort, nlong - base);
-            for (int t = lane; t < cnt; t += 32) {
-                int pe = e_long ? base + t : t;
-                int pi = e_long ? t : base + t;
-                int se = m.eperm[pe], si = m.iperm[pi];
-                real4 A = m.eu[se], B = m.iu[si];
-                real q = (real)(m.ist[si] & 0xff) + B.w;
-                real npair = e_long ? n_i * r_fmax(A.w, wi) / wi : n_e * r_fmax(A.w, wi) / A.w;
-                U4 r = e_long ? draw(seed, m.eid[pe], step, PU_COLL_EI)
-                              : draw(seed, (unsigned long long)m.iid[pi], step, PU_COLL_IE);
-                real3 ua = make_real3(A.x, A.y, A.z), ub = make_real3(B.x, B.y, B.z);
-                if (binary_collision(ua, ub, RF(1.0), mi, -RF(1.0), q, A.w, wi, npair, lnL, S.dt,
-                                     u01(r.x), u01(r.y), u01(r.z), u01(r.w))) c_ei++;
-                m.eu[se] = make_real4(ua.x, ua.y, ua.z, A.w);
-                m.iu[si] = make_real4(ub.x, ub.y, ub.z, B.w);
+        // the longer species in order, the shorter cycled: particle t of the
+        // shorter meets t, t + nshort, ... of the longer, one after another,
+        // and no other thread touches any of them
+        if (ne >= ni) {
+            for (int pi = t0; pi < ni; pi += nt) {
+                real4 B = m.iu[pi];
+                const real q = (real)(m.ist[pi] & 0xff) + B.w;
+#pragma unroll 1
+                for (int pe = pi; pe < ne; pe += ni) {
+                    const real4 A = m.eu[pe];
+                    const real npair = n_i * r_fmax(A.w, wi) / wi;
+                    const U4 r = draw(seed, m.eid[pe], step, PU_COLL_EI);
+                    const Collided c = binary_collision(A, B, RF(1.0), mi, -RF(1.0), q, A.w, wi, npair, lnL, dt, r);
+                    lt.ei += c.hit;
+                    m.eu[pe] = c.a;
+                    B = c.b;
+                }
+                m.iu[pi] = B;
             }
-            __syncwarp();
+        } else {
+            for (int pe = t0; pe < ne; pe += nt) {
+                real4 A = m.eu[pe];
+#pragma unroll 1
+                for (int pi = pe; pi < ni; pi += ne) {
+                    const real4 B = m.iu[pi];
+                    const real q = (real)(m.ist[pi] & 0xff) + B.w;
+                    const real npair = n_e * r_fmax(A.w, wi) / A.w;
+                    const U4 r = draw(seed, (unsigned long long)m.iid[pi], step, PU_COLL_IE);
+                    const Collided c = binary_collision(A, B, RF(1.0), mi, -RF(1.0), q, A.w, wi, npair, lnL, dt, r);
+                    lt.ei += c.hit;
+                    A = c.a;
+                    m.iu[pi] = c.b;
+                }
+                m.eu[pe] = A;
+            }
         }
+        team_sync<TW>();
     }
     if (coll && ne >= 1) {
-        dd pk = dd_zero(), pki = dd_zero();
-        for (int k = lane; k < ne; k += 32) { real4 u = m.eu[m.eperm[k]]; pk = dd_addf(pk, u.w * MC2 * gm1(u.x, u.y, u.z)); }
-        for (int k = lane; k < ni; k += 32) { real4 u = m.iu[m.iperm[k]]; pki = dd_addf(pki, wi * MC2 * mi * gm1(u.x, u.y, u.z)); }
-        dd Ke = wsum_dd(pk), Ki = wsum_dd(pki);
+        // kinetic energies after the collisions; each electron's gamma - 1
+        // stays in the scratch for the passes below
+        dd Ke = dd_zero(), Ki = dd_zero();
+        if constexpr (TW == 1) {
+            for (int k = lane; k < ne; k += 32) {
+                const real4 u = m.eu[k];
+                const real g1 = gm1(u.x, u.y, u.z);
+                m.ew[k].x = g1;
+                Ke = dd_addp(Ke, r_mul(u.w, MC2), g1);
+            }
+            for (int k = lane; k < ni; k += 32) { real4 u = m.iu[k]; Ki = dd_addp(Ki, mw_i, gm1(u.x, u.y, u.z)); }
+            wsum_dd2(Ke, Ki, lane);
+        } else {
+            for (int k = t0; k < ne; k += nt) { const real4 u = m.eu[k]; m.ew[k].x = gm1(u.x, u.y, u.z); }
+            __syncthreads();
+            if (w0) {
+                for (int k = lane; k < ne; k += 32) Ke = dd_addp(Ke, r_mul(m.eu[k].w, MC2), m.ew[k].x);
+                Ke = wsum_dd(Ke);
+                if (lane == 0) m.bc[0] = Ke;
+            }
+            if (w1) {
+                for (int k = lane; k < ni; k += 32) { real4 u = m.iu[k]; Ki = dd_addp(Ki, mw_i, gm1(u.x, u.y, u.z)); }
+                Ki = wsum_dd(Ki);
+                if (lane == 0) m.bc[1] = Ki;
+            }
+            __syncthreads();
+            Ke = m.bc[0]; Ki = m.bc[1];
+        }
         real ke = dd_f(Ke);
         real delta = RF(0.0);
         if (ke > RF(0.0)) {
@@ -695,64 +807,72 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
         }
         if ((flags & 4u) && ni >= 1) {
             // the restore and the ionization stage's per-electron inputs in
-            // one pass: kinetic energy and w * beta after the restore, in
-            // the sort-key storage (free until recombination), and their sum
-            real2 *ew = reinterpret_cast<real2 *>(m.ekey);
+            // one pass: kinetic energy and w * beta after the restore, and
+            // the kinetic energies' sum
             dd pt = dd_zero();
-            for (int k = lane; k < ne; k += 32) {
-                const int sl = m.eperm[k];
-                real4 u = m.eu[sl];
-                scale_kinetic(u.x, u.y, u.z, delta);
-                m.eu[sl] = u;
-                real u2 = u.x * u.x + u.y * u.y + u.z * u.z;
-                real g1 = u2 / (r_sqrt(RF(1.0) + u2) + RF(1.0));
-                pt = dd_addf(pt, u.w * MC2 * g1);
-                ew[k] = make_real2(MC2 * g1, u.w * (r_sqrt(u2) / (RF(1.0) + g1)));
+            for (int k = t0; k < ne; k += nt) {
+                real4 u = m.eu[k];
+                scale_kinetic(u.x, u.y, u.z, m.ew[k].x, delta);
+                m.eu[k] = u;
+                real u2 = square3_yx(u.x, u.y, u.z);
+                real g1 = gm1_of(u2);
+                if constexpr (TW == 1) pt = dd_addp(pt, r_mul(u.w, MC2), g1);
+                m.ew[k] = make_real2(MC2 * g1, u.w * (r_sqrt(u2) / (RF(1.0) + g1)));
             }
-            Kt = wsum_dd(pt);
+            if constexpr (TW == 1) Kt = wsum_dd(pt);
             ew_ready = true;
         } else if (delta != RF(0.0)) {
-            for (int k = lane; k < ne; k += 32) {
+            for (int k = t0; k < ne; k += nt) {
                 real4 u = m.eu[k];
-                scale_kinetic(u.x, u.y, u.z, delta);
+                scale_kinetic(u.x, u.y, u.z, m.ew[k].x, delta);
                 m.eu[k] = u;
             }
         }
-        __syncwarp();
+        team_sync<TW>();
     }
 
     }
-    __syncthreads();
+    if constexpr (TW == 1) __syncthreads();
 
     if (on) {
     // ---- Lotz impact ionization, cell-average probability (Eq. 3) ----
     if ((flags & 4u) && ne >= 1 && ni >= 1) {
+        // charge states present (every warp of a team for itself)
         unsigned pmask = 0;
         for (int k = lane; k < ni; k += 32) { int Z = m.ist[k] & 0xff; if (Z < ZNUC) pmask |= 1u << Z; }
-        for (int o = 16; o > 0; o >>= 1) pmask |= __shfl_xor_sync(FULL, pmask, o);
-        // kinetic energy and w * beta of each electron (canonical order), kept
-        // in the sort-key storage, which is free until recombination
-        real2 *ew = reinterpret_cast<real2 *>(m.ekey);
-        int nhot;
+        pmask = __reduce_or_sync(FULL, pmask);
+        // kinetic energy and w * beta of each electron (canonical order)
+        real2 *ew = m.ew;
+        int nhot = 0;
         if (!ew_ready) {
             dd pk = dd_zero();
-            for (int k = lane; k < ne; k += 32) {
-                real4 u = m.eu[m.eperm[k]];
-                real u2 = u.x * u.x + u.y * u.y + u.z * u.z;
-                real g1 = u2 / (r_sqrt(RF(1.0) + u2) + RF(1.0));
-                pk = dd_addf(pk, u.w * MC2 * g1);
+            for (int k = t0; k < ne; k += nt) {
+                real4 u = m.eu[k];
+                real u2 = square3(u.x, u.y, u.z);
+                real g1 = gm1_of(u2);
+                if constexpr (TW == 1) pk = dd_addp(pk, r_mul(u.w, MC2), g1);
                 ew[k] = make_real2(MC2 * g1, u.w * (r_sqrt(u2) / (RF(1.0) + g1)));
             }
-            Kt = wsum_dd(pk);
+            if constexpr (TW == 1) Kt = wsum_dd(pk);
+            team_sync<TW>();
         }
-        __syncwarp();
         // Electrons at or below the lowest lowered binding of every charge
         // state present ionize nothing and add nothing to the sums: the
         // others (a hot tail, typically a few per cent) are gathered in
         // canonical order to the front of the storage, so that a warp's
         // lanes do not idle beside the one lane with a hot electron.
-        nhot = ne;
-        {
+        if (TW > 1 && w1) {
+            dd pt = dd_zero();
+            for (int k = lane; k < ne; k += 32) {
+                const real4 u = m.eu[k];
+                real u2 = ew_ready ? square3_yx(u.x, u.y, u.z) : square3(u.x, u.y, u.z);
+                real g1 = gm1_of(u2);
+                pt = dd_addp(pt, r_mul(u.w, MC2), g1);
+            }
+            pt = wsum_dd(pt);
+            if (lane == 0) m.bc[2] = pt;
+        }
+        if (w0) {
             real Pall = RF(3.0e38);
             for (int z = 0; z < ZNUC; ++z) {
                 if (!(pmask & (1u << z))) continue;
@@ -760,7 +880,8 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
                     Pall = r_fmin(Pall, lowered_binding(T, z, lane, m.dE[z]));
             }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) Pall = r_fmin(Pall, __shfl_xor_sync(FULL, Pall, o));
+            for (int o = 4; o > 0; o >>= 1) Pall = r_fmin(Pall, __shfl_xor_sync(FULL, Pall, o));
+            Pall = __shfl_sync(FULL, Pall, 0);
             int nh = 0;
             for (int b0 = 0; b0 < ne; b0 += 32) {
                 const int k = b0 + lane;
@@ -773,10 +894,19 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
                 __syncwarp();
             }
             nhot = nh;
+            if (TW > 1 && lane == 0) m.bc[3].hi = (real)nh;
         }
-        const real cfac = (real)(kCcmPerFs) * S.dt * nref;
+        if constexpr (TW > 1) {
+            __syncthreads();
+            Kt = m.bc[2];
+            nhot = (int)m.bc[3].hi;
+        }
+        const real cfac = (real)(kCcmPerFs) * dt * nref;
+        real4 *lz = m.lz + (TW == 1 ? 0 : warp * NS);
+        int zi = 0;
         for (int z = 0; z < ZNUC; ++z) {
             if (!(pmask & (1u << z))) continue;
+            if (TW > 1 && (zi++ % TW) != warp) continue;
             // Lotz constants of charge state z (lowest-energy configuration):
             // lowered binding P, 1/P, ln P, a * occupation (0: empty subshell)
             if (lane < NS) {
@@ -786,7 +916,7 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
                     const real P = lowered_binding(T, z, lane, m.dE[z]);
                     v = make_real4(P, RF(1.0) / P, r_log(P), T.lotz_a[lane] * (real)o);
                 }
-                m.lz[lane] = v;
+                lz[lane] = v;
             }
             __syncwarp();
             // the lowest lowered binding of the charge state: electrons at
@@ -794,7 +924,7 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
             real Pmin = RF(3.0e38);
 #pragma unroll
             for (int sh = 0; sh < NS; ++sh)
-                if (m.lz[sh].w > RF(0.0)) Pmin = r_fmin(Pmin, m.lz[sh].x);
+                if (lz[sh].w > RF(0.0)) Pmin = r_fmin(Pmin, lz[sh].x);
             // fast log / exp: a few ulp on a probability; only a decision
             // within that of its threshold could flip
             dd pr = dd_zero();
@@ -805,7 +935,7 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
                 real sig = RF(0.0);
 #pragma unroll
                 for (int sh = 0; sh < NS; ++sh) {
-                    const real4 L = m.lz[sh];
+                    const real4 L = lz[sh];
                     if (L.w > RF(0.0) && E > L.x) {
                         const real x = E * L.y;
                         sig += L.w * (lnE - L.z) * (invE * L.y) *
@@ -814,102 +944,136 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
                 }
                 pr = dd_addf(pr, q.y * sig);
             }
-            real P = cfac * dd_f(wsum_dd(pr));
+            // no hot electron: the sum is zero
+            real P = nhot > 0 ? cfac * dd_f(wsum_dd(pr)) : RF(0.0);
             if (lane == 0) m.Pz[z] = P;
             if (P > RF(1.0) && lane == 0) wt.cnt[C_PGT1]++;
             __syncwarp();
         }
-        __syncwarp();
-        dd carry = dd_zero(), paid = dd_zero();
-        for (int b0 = 0; b0 < ni; b0 += 32) {
-            int t = b0 + lane;
-            bool cand = false;
-            real cost = RF(0.0);
-            int sl = 0, Z = 0, nK = 0;
-            if (t < ni) {
-                sl = m.iperm[t];
-                int st = m.ist[sl];
-                Z = st & 0xff; nK = (st >> 8) & 0xff;
-                if (Z < ZNUC) {
-                    U4 r = draw(seed, (unsigned long long)m.iid[t], step, PU_ION);
-                    if (u01(r.x) < m.Pz[Z]) {
-                        cand = true;
-                        cost = wi * removal_energy(T, Z, nK, m.dE[Z]);
+        team_sync<TW>();
+        dd paid = dd_zero();
+        if (w0) {
+            dd carry = dd_zero();
+            for (int b0 = 0; b0 < ni; b0 += 32) {
+                int t = b0 + lane;
+                bool cand = false;
+                real cost = RF(0.0);
+                int Z = 0, nK = 0;
+                if (t < ni) {
+                    int st = m.ist[t];
+                    Z = st & 0xff; nK = (st >> 8) & 0xff;
+                    if (Z < ZNUC) {
+                        U4 r = draw(seed, (unsigned long long)m.iid[t], step, PU_ION);
+                        if (u01(r.x) < m.Pz[Z]) {
+                            cand = true;
+                            cost = wi * removal_energy(T, Z, nK, m.dE[Z]);
+                        }
                     }
                 }
-            }
-            dd incl = dd_add(carry, wscan_dd(dd{cost, RF(0.0)}, lane));
-            bool acc = cand && dd_le(incl, Kt);
-            if (cand && !acc) c_rej++;
-            unsigned bal = __ballot_sync(FULL, acc);
-            if (acc) {
-                int so = outer_shell(ZNUC - Z, nK);
-                lose_electron(Z, nK, so);
-                m.ist[sl] = Z | (nK << 8);
-                int pos = nnew + __popc(bal & ((1u << lane) - 1u));
-                if (pos < a.cap_new) {
-                    NewE q; q.ux = q.uy = q.uz = RF(0.0); q.w = wi; q.meta = sl | (KIND_IMPACT << 16);
-                    m.nw[pos] = q;
-                } else {
-                    atomicOr(a.err, ERR_NEW_OVERFLOW);
+                // no candidate among these ions (most cells): nothing to pay
+                if (!__any_sync(FULL, cand)) continue;
+                dd incl = dd_add(carry, wscan_dd(dd{cost, RF(0.0)}, lane));
+                bool acc = cand && dd_le(incl, Kt);
+                if (cand && !acc) lt.rej++;
+                unsigned bal = __ballot_sync(FULL, acc);
+                if (acc) {
+                    int so = outer_shell(ZNUC - Z, nK);
+                    lose_electron(Z, nK, so);
+                    m.ist[t] = Z | (nK << 8);
+                    int pos = nnew + __popc(bal & ((1u << lane) - 1u));
+                    if (pos < a.cap_new) {
+                        NewE q; q.ux = q.uy = q.uz = RF(0.0); q.w = wi; q.meta = t | (KIND_IMPACT << 16);
+                        m.nw[pos] = q;
+                    } else {
+                        atomicOr(a.err, ERR_NEW_OVERFLOW);
+                    }
+                    lt.ion++;
                 }
-                c_ion++;
+                paid = dd_add(paid, wsum_dd(dd{acc ? cost : RF(0.0), RF(0.0)}));
+                nnew += __popc(bal);
+                n_imp += __popc(bal);
+                carry = wlane_dd(incl, 31);
             }
-            paid = dd_add(paid, wsum_dd(dd{acc ? cost : RF(0.0), RF(0.0)}));
-            nnew += __popc(bal);
-            n_imp += __popc(bal);
-            carry = wbcast_dd(incl, 31);
+            nnew = min(nnew, a.cap_new);
+            if (TW > 1 && lane == 0) m.bc[4] = paid;
         }
-        nnew = min(nnew, a.cap_new);
+        if constexpr (TW > 1) {
+            __syncthreads();
+            paid = m.bc[4];
+        }
         Wnew_imp = nnew * wi;
         paid_cell = paid;
         ionized = true;
         real pf = dd_f(paid);
         if (pf > RF(0.0)) {
             real delta = pf / dd_f(Kt);
-            for (int k = lane; k < ne; k += 32) {
+            for (int k = t0; k < ne; k += nt) {
                 real4 u = m.eu[k];
-                scale_kinetic(u.x, u.y, u.z, delta);
+                scale_kinetic(u.x, u.y, u.z, gm1(u.x, u.y, u.z), delta);
                 m.eu[k] = u;
             }
-            wt.ion = dd_add(wt.ion, paid);
+            if (w0) wt.ion = dd_add(wt.ion, paid);
         }
-        __syncwarp();
+        team_sync<TW>();
     }
 
     }
-    __syncthreads();
+    if constexpr (TW == 1) __syncthreads();
 
     if (on) {
-    CellCtx cc;
-    cc.s = s; cc.lc = lc; cc.cx = cx; cc.cy = cy; cc.e0 = e0; cc.ne = ne; cc.i0 = i0; cc.ni = ni;
-    cc.step = step; cc.flags = flags; cc.seed = seed; cc.wi = wi; cc.mi = mi; cc.n_e = n_e; cc.n_i = n_i;
-    cc.nref = nref; cc.rad = rad;
-    cc.have_sums = all_bulk && ionized;
-    cc.K_after = dd_sub(Kt, paid_cell);
-    cc.W_e = We_cell;
-    cc.Q_after = dd_f(Qcell) + (real)n_imp;
-    if ((flags & 8u) && ni >= 1) stage_recombine(a, m, T, S, cc, lane, Wnew_imp, wt);
-    if (rad && (flags & 16u) && S.nb && ni >= 1) stage_photo(a, m, T, S, cc, lane, nnew, wt);
-    if (rad && (flags & 32u) && ni >= 1) stage_decay(a, m, T, S, cc, lane, nnew, wt);
-    if (rad && (flags & 256u)) stage_therm(a, m, cc, lane, nnew);
+    if ((flags & 8u) && ni >= 1) {
+        CellCtx cc;
+        cc.lc = lc; cc.ne = ne; cc.ni = ni;
+        cc.step = step; cc.seed = seed; cc.wi = wi; cc.n_i = n_i; cc.nref = nref;
+        cc.have_sums = all_bulk && ionized;
+        cc.K_after = dd_sub(Kt, paid_cell);
+        cc.W_e = We_cell;
+        cc.Q_after = dd_f(Qcell) + (real)n_imp;
+        real delta = RF(0.0);
+        bool rec = false;
+        if (w0) {
+            rec = stage_recombine(a, m, T, S, cc, lane, Wnew_imp, wt, delta);
+            if (TW > 1 && lane == 0) m.bc[5] = dd{delta, rec ? RF(1.0) : RF(0.0)};
+        }
+        if constexpr (TW > 1) {
+            __syncthreads();
+            delta = m.bc[5].hi;
+            rec = m.bc[5].lo != RF(0.0);
+        }
+        if (rec) recombine_apply(m, S, ne, delta, t0, nt);
+        team_sync<TW>();
+    }
+    if (rad && w0) {
+        CellCtx cc;
+        cc.lc = lc; cc.ne = ne; cc.ni = ni;
+        cc.step = step; cc.seed = seed; cc.wi = wi; cc.n_i = n_i; cc.nref = nref;
+        if ((flags & 16u) && S.nb && ni >= 1) stage_photo(a, m, T, S, cc, lane, nnew, wt);
+        if ((flags & 32u) && ni >= 1) stage_decay(a, m, T, S, cc, lane, nnew, wt);
+        if (flags & 256u) stage_therm(m, cc, lane, nnew);
+    }
+    if (TW > 1 && rad) __syncthreads();
 
     // ---- write the collided state back, each cell's records in its
     //      canonical order (the order the push kernel follows) ----
-    for (int k = lane; k < ne; k += 32) {
-        const int sl = m.eperm[k];
-        const real4 u = m.eu[sl];
-        const real2 x = m.epos[sl];
+    for (int k = t0; k < ne; k += nt) {
+        const real4 u = m.eu[k];
+        const real2 x = m.epos[k];
         a.e0[e0 + k] = make_real4(x.x, x.y, u.x, u.y);
         a.e1[e0 + k] = rec_e1(u.z, u.w, m.eid[k]);
     }
-    if (rad && S.rt) {
+    for (int k = t0; k < ni; k += nt) {
+        const real4 u = m.iu[k];
+        const real2 x = m.ipos[k];
+        a.i0[i0 + k] = make_real4(x.x, x.y, u.x, u.y);
+        a.i1[i0 + k] = rec_i1(u.z, u.w, m.iid[k], m.ist[k]);
+    }
+    if (rad && S.rt && w0) {
         // transport mode: the cell's electron weight after the step, created
         // electrons included: its share of the next heating of its rad cell
         // (summed in canonical order: the slots' order is the scatter's)
         real wsum = RF(0.0);
         for (int k = lane; k < ne; k += 32) {
-            const real w = m.eu[m.eperm[k]].w;
+            const real w = m.eu[k].w;
             wsum += w > RF(0.0) ? w : RF(0.0);
         }
         for (int k = lane; k < nnew; k += 32) wsum += m.nw[k].w;
@@ -917,7 +1081,7 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
         if (lane == 0) S.rt_w[lc] = (float)wsum;
     }
     // ---- created electrons: after the sorted range, at their ion, with their cell as key ----
-    if (nnew > 0) {
+    if (w0 && nnew > 0) {
         // a slab with a budget of its own keeps its electrons within it: a
         // cell that would take it beyond drops what it created and fails
         // the slab alone (it is stopped at the end of the step); the others
@@ -944,87 +1108,80 @@ __device__ void process_round(const CellArgs &a, const WarpMem &m, const Tables 
         }
         for (int k = lane; k < n_ok; k += 32) {
             NewE q = m.nw[k];
-            int islot = q.meta & 0xffff, kind = q.meta >> 16;
-            real4 I0 = a.i0[i0 + islot];
-            real4 I1 = a.i1[i0 + islot];
+            const int ip = q.meta & 0xffff, kind = q.meta >> 16;
+            const real2 x = m.ipos[ip];
             unsigned idhi = ((step + 1u) << 2) | (unsigned)kind;
-            a.e0[sorted + base + k] = make_real4(I0.x, I0.y, q.ux, q.uy);
-            a.e1[sorted + base + k] = rec_e1(q.uz, q.w, ((unsigned long long)idhi << 32) | rec_iid(I1));
+            a.e0[sorted + base + k] = make_real4(x.x, x.y, q.ux, q.uy);
+            a.e1[sorted + base + k] = rec_e1(q.uz, q.w, ((unsigned long long)idhi << 32) | m.iid[ip]);
             a.ekey[sorted + base + k] = g;
         }
     }
-    __syncwarp();
-    // ions last: the created electrons above read their parent ions' records
-    // at the ions' slots
-    for (int k = lane; k < ni; k += 32) {
-        const int sl = m.iperm[k];
-        const real4 u = m.iu[sl];
-        const real2 x = m.ipos[sl];
-        a.i0[i0 + k] = make_real4(x.x, x.y, u.x, u.y);
-        a.i1[i0 + k] = rec_i1(u.z, u.w, m.iid[k], m.ist[sl]);
-    }
-
-    // ---- tallies (lane-uniform) ----
-    wt.cnt[C_EE] += wsum_i(c_ee);
-    wt.cnt[C_EI] += wsum_i(c_ei);
-    wt.cnt[C_ION] += wsum_i(c_ion);
-    wt.cnt[C_ION_REJ] += wsum_i(c_rej);
-    __syncwarp();
     }
     __syncthreads();
 }
 
-// Each round the block takes one cell per warp from a shared counter.
+// Bound by instruction issue and the latency of dependent chains at 16
+// resident warps per SM (128 registers); its memory side moves only the 64 B
+// per particle.  So it is written for few instructions per particle: the
+// order sorts 32-bit words, the records are staged in that order (no index
+// loads, no bank conflicts), up to four cell sums share one reduction, each
+// electron's gamma - 1 is kept between the collision restore's two passes,
+// the collisions are inline with their particles in registers, and an ion
+// keeps its state in registers through its chain of collisions.  Against the
+// 64-bit sort, slot-ordered staging, one reduction per sum and collisions
+// called by reference: 2048 x 256 cells of 64 e + 16 i, 42 M particles, 6.94
+// -> 5.40 ms a step; 512 x 64 cells 511 -> 397 us.
+// Each round the block takes one cell per team from a shared counter.
 // Cells whose population exceeds this launch's shared-memory capacity go to
-// a list for the large-cell launch.
-// RMAX: the largest cell sorted in registers (128: launches whose staging
-// holds at most 128 entries per species; 512: up to 512; 1024: the launches
-// for larger cells, with up to 255 registers a thread for the 32-entry
-// register sort, radix-sorting cells above 1024).
-template <int RMAX>
-__global__ void __launch_bounds__(RMAX > 512 ? 128 : 256, RMAX > 512 ? 1 : 2) k_cell(CellArgs a)
+// a list for the next launch.
+// RMAX: the most entries per species a launch stages; TW: warps per cell.
+template <int RMAX, int TW>
+__global__ void __launch_bounds__(TW == 1 ? 256 : 32 * TW, TW == 1 ? 2 : 4) k_cell(CellArgs a)
 {
     extern __shared__ __align__(kSmAlign) char smem[];
     __shared__ Tables T;
     __shared__ int round_base;
     for (int k = threadIdx.x; k < (int)(sizeof(Tables) / sizeof(real)); k += blockDim.x)
         ((real *)&T)[k] = ((const real *)a.tab)[k];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const size_t gwarp = (size_t)blockIdx.x * nwarp + warp;
-    WarpMem m = carve(smem + (size_t)warp * warp_mem_bytes(a.cap_ce, a.cap_ci), a.cap_ce, a.cap_ci,
-                      a.nw + gwarp * a.cap_new, a.gw + gwarp * warp_gmem_words(a.cap_ce, a.cap_ci));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nteam = TW == 1 ? blockDim.x >> 5 : 1;
+    const int team = TW == 1 ? warp : 0;
+    CellMem m = carve(smem + (size_t)team * cell_mem_bytes(a.cap_ce, a.cap_ci), a.cap_ce, a.cap_ci,
+                      a.nw + ((size_t)blockIdx.x * nteam + team) * a.cap_new);
     const int total = a.list ? *a.n_list : a.ncell;
     WarpTally wt;
+    LaneTally lt{0, 0, 0, 0};
     wt.slab = -1;
     wt.ion = wt.ka = wt.esc = wt.rt = dd_zero();
     for (int q = 0; q < NCOUNT; ++q) wt.cnt[q] = 0;
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) round_base = atomicAdd(a.work, nwarp);
+        if (threadIdx.x == 0) round_base = atomicAdd(a.work, nteam);
         __syncthreads();
         const int base = round_base;
         if (base >= total) break;
         int g = -1;
-        if (base + warp < total) {
-            g = a.list ? a.list[base + warp] : base + warp;
+        if (base + team < total) {
+            g = a.list ? a.list[base + team] : base + team;
             int ne = a.cs_e[g + 1] - a.cs_e[g], ni = a.cs_i[g + 1] - a.cs_i[g];
             if (ne > a.cap_ce || ni > a.cap_ci || 3 * ni > a.cap_new) {
-                if (a.ovf_list) {
-                    if (lane == 0) a.ovf_list[atomicAdd(a.ovf_count, 1)] = g;
-                } else {
-                    // no larger pass left: report, and drop the cell's particles so
-                    // that the next sort stays consistent
-                    if (lane == 0) atomicOr(a.err, ERR_CELL_OVERFLOW);
-                    for (int k = a.cs_e[g] + lane; k < a.cs_e[g + 1]; k += 32)
-                        reinterpret_cast<real *>(a.e1 + k)[1] = RF(0.0);
-                    for (int k = a.cs_i[g] + lane; k < a.cs_i[g + 1]; k += 32) a.i1[k].w = bits_real(0xffu);
+                if (TW == 1 || warp == 0) {
+                    if (a.ovf_list) {
+                        if (lane == 0) a.ovf_list[atomicAdd(a.ovf_count, 1)] = g;
+                    } else {
+                        // no larger pass left: report, and drop the cell's particles so
+                        // that the next sort stays consistent
+                        if (lane == 0) atomicOr(a.err, ERR_CELL_OVERFLOW);
+                        for (int k = a.cs_e[g] + lane; k < a.cs_e[g + 1]; k += 32)
+                            reinterpret_cast<real *>(a.e1 + k)[1] = RF(0.0);
+                        for (int k = a.cs_i[g] + lane; k < a.cs_i[g + 1]; k += 32) a.i1[k].w = bits_real(0xffu);
+                    }
                 }
                 g = -1;
             }
         }
-        process_round<RMAX>(a, m, T, g, lane, wt);
+        process_cell<RMAX, TW>(a, m, T, g, warp, lane, wt, lt);
     }
-    tally_flush(a, wt, lane);
+    tally_flush(a, wt, lt, lane);
 }
 
 }  // namespace pic

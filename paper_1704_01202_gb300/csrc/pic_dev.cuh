@@ -40,6 +40,8 @@ struct real3 { double x, y, z; };
 #define r_cbrt cbrt
 #define r_pow pow
 #define r_fma fma
+#define r_mul __dmul_rn
+#define r_add __dadd_rn
 #else
 typedef float real;
 typedef float4 real4;
@@ -63,6 +65,8 @@ typedef float3 real3;
 #define r_cbrt cbrtf
 #define r_pow powf
 #define r_fma fmaf
+#define r_mul __fmul_rn
+#define r_add __fadd_rn
 #endif
 __host__ __device__ __forceinline__ real4 make_real4(real x, real y, real z, real w)
 {
@@ -124,6 +128,10 @@ __host__ __device__ __forceinline__ int rec_ist(const real4 &p1) { return (int)(
 __host__ __device__ __forceinline__ real4 rec_i1(real uz, real zf, uint32_t id, int st)
 {
     return make_real4(uz, zf, bits_real(id), bits_real((uint32_t)st));
+}
+__device__ __forceinline__ void prefetch_l2(const void *p)
+{
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 // largest value below 1 (positions inside a cell stay < 1)
 constexpr real kBelow1 = sizeof(real) == 8 ? (real)0.99999999999999989 : (real)0.99999994f;
@@ -356,6 +364,16 @@ __device__ __forceinline__ dd dd_add(dd a, dd b)
     return dd{h, e - (h - s)};
 }
 __device__ __forceinline__ dd dd_addf(dd a, real b) { return dd_add(a, dd{b, RF(0.0)}); }
+// a + x y, the product unrounded
+__device__ __forceinline__ dd dd_addp(dd a, real x, real y)
+{
+    real s = r_fma(x, y, a.hi);
+    real bv = s - a.hi;
+    real e = (a.hi - (s - bv)) + r_fma(x, y, -bv);
+    e += a.lo;
+    real h = s + e;
+    return dd{h, e - (h - s)};
+}
 __device__ __forceinline__ dd dd_neg(dd a) { return dd{-a.hi, -a.lo}; }
 __device__ __forceinline__ dd dd_sub(dd a, dd b) { return dd_add(a, dd_neg(b)); }
 __device__ __forceinline__ real dd_f(dd a) { return a.hi + a.lo; }
@@ -396,97 +414,126 @@ __device__ __forceinline__ real eos_lookup(const EosTable &T, real n, real t)
 
 // ---------------- kinematics ----------------
 // kinetic energy in units of m c^2 (gamma - 1 = u^2 / (gamma + 1))
-__device__ __forceinline__ real gm1(real ux, real uy, real uz)
+__device__ __forceinline__ real square3(real ux, real uy, real uz)
 {
-    real u2 = ux * ux + uy * uy + uz * uz;
-    return u2 / (r_sqrt(RF(1.0) + u2) + RF(1.0));
+    return r_fma(uz, uz, r_fma(ux, ux, r_mul(uy, uy)));
 }
+// the same with the x and y products exchanged in the roundings
+__device__ __forceinline__ real square3_yx(real ux, real uy, real uz)
+{
+    return r_fma(uz, uz, r_fma(uy, uy, r_mul(ux, ux)));
+}
+__device__ __forceinline__ real gm1_of(real u2) { return u2 / (r_sqrt(RF(1.0) + u2) + RF(1.0)); }
+__device__ __forceinline__ real gm1(real ux, real uy, real uz) { return gm1_of(square3(ux, uy, uz)); }
 
 // Multiply the kinetic energy of u by f = 1 - delta, direction kept.  The
 // factor is carried as delta and 1 - |u'|/|u| is formed without
 // cancellation, so small corrections are not lost to FP32 rounding of f.
-__device__ __forceinline__ void scale_kinetic(real &ux, real &uy, real &uz, real delta)
+// g1: gamma - 1 of u.
+__device__ __forceinline__ void scale_kinetic(real &ux, real &uy, real &uz, real g1, real delta)
 {
-    real g1 = gm1(ux, uy, uz);
     if (g1 == RF(0.0) || delta == RF(0.0)) return;
     real b = delta * g1 / (RF(2.0) + g1);
     real x = delta + b - delta * b;                   // 1 - (|u'|/|u|)^2
     real d = x / (RF(1.0) + r_sqrt(RF(1.0) - x));            // 1 - |u'|/|u|
     ux -= ux * d; uy -= uy * d; uz -= uz * d;
 }
+__device__ __forceinline__ void scale_kinetic(real &ux, real &uy, real &uz, real delta)
+{
+    scale_kinetic(ux, uy, uz, gm1(ux, uy, uz), delta);
+}
 
 // One binary collision: Takizuka-Abe deflection tan(theta/2) ~ N(0, var),
 // var = 2 pi (qa qb)^2 r_e^2 c n lnL dt / (mu^2 beta_rel^3), applied as a
 // rotation of the centre-of-momentum momentum; weighted acceptance
-// min(1, w_other / w_self).  Masses in m_e, u in units of m c of each.
-__device__ __noinline__ bool binary_collision(real3 &ua, real3 &ub, real ma, real mb, real qa, real qb,
-                                                 real wa, real wb, real n_l, real lnL, real dtc,
-                                                 real r0, real r1, real r2, real r3)
+// min(1, w_other / w_self).  Masses in m_e, u in units of m c of each; the
+// fourth component of a particle passes through.  The particles go in and
+// come back by value, in registers.
+//
+// The products that are fused into a sum are written out (r_fma; r_mul and
+// r_add are never contracted): a cell's events follow from the last bits of
+// its momenta, so the rounding may not depend on what the compiler fuses
+// where the function is called.
+struct Collided { real4 a, b; int hit; };
+
+__device__ __forceinline__ real dot3(real ax, real ay, real az, real bx, real by, real bz)
 {
-    if (qa == RF(0.0) || qb == RF(0.0)) return false;
+    return r_fma(az, bz, r_fma(ax, bx, r_mul(ay, by)));
+}
+
+__device__ __forceinline__ Collided binary_collision(real4 ua, real4 ub, real ma, real mb, real qa, real qb,
+                                                     real wa, real wb, real n_l, real lnL, real dtc, U4 rnd)
+{
+    if (qa == RF(0.0) || qb == RF(0.0)) return Collided{ua, ub, 0};
+    const real r0 = u01(rnd.x), r1 = u01(rnd.y), r2 = u01(rnd.z), r3 = u01(rnd.w);
     // divisions by the same quantity are done once, as a reciprocal
-    real ga = r_sqrt(RF(1.0) + ua.x * ua.x + ua.y * ua.y + ua.z * ua.z);
-    real gb = r_sqrt(RF(1.0) + ub.x * ub.x + ub.y * ub.y + ub.z * ub.z);
+    const real ga = r_sqrt(r_fma(ua.z, ua.z, r_fma(ua.y, ua.y, r_fma(ua.x, ua.x, RF(1.0)))));
+    const real gb = r_sqrt(r_fma(ub.z, ub.z, r_fma(ub.y, ub.y, r_fma(ub.x, ub.x, RF(1.0)))));
     const real iga = RF(1.0) / ga, igb = RF(1.0) / gb;
-    real dvx = ua.x * iga - ub.x * igb, dvy = ua.y * iga - ub.y * igb, dvz = ua.z * iga - ub.z * igb;
-    real vrel = r_sqrt(dvx * dvx + dvy * dvy + dvz * dvz);
-    if (vrel < RF(1e-10)) return false;
-    real mu = ma * mb / (ma + mb);
+    const real dvx = r_fma(ua.x, iga, -r_mul(ub.x, igb)), dvy = r_fma(ua.y, iga, -r_mul(ub.y, igb)),
+               dvz = r_fma(ua.z, iga, -r_mul(ub.z, igb));
+    const real vrel = r_sqrt(dot3(dvx, dvy, dvz, dvx, dvy, dvz));
+    if (vrel < RF(1e-10)) return Collided{ua, ub, 0};
+    const real mu = r_mul(ma, mb) / r_add(ma, mb);
     // constant part 2 pi r_e^2 c in cm^3/fs, evaluated in double once
     const real k0 = (real)(2.0 * kPi * kReCm * kReCm * kCcmPerFs);
-    real q2 = qa * qb;
-    real var = k0 * q2 * q2 * n_l * lnL * dtc / (mu * mu * vrel * vrel * vrel);
-    real delta = r_sqrt(var) * r_sqrt(-RF(2.0) * r_log(r0)) * r_cospi(RF(2.0) * r1);
+    const real q2 = r_mul(qa, qb);
+    const real var = r_mul(r_mul(r_mul(r_mul(r_mul(k0, q2), q2), n_l), lnL), dtc) /
+                     r_mul(r_mul(r_mul(r_mul(mu, mu), vrel), vrel), vrel);
+    const real delta = r_mul(r_mul(r_sqrt(var), r_sqrt(r_mul(-RF(2.0), r_log(r0)))), r_cospi(r_mul(RF(2.0), r1)));
     real sphi, cphi;
-    r_sincospi(RF(2.0) * r2, &sphi, &cphi);
+    r_sincospi(r_mul(RF(2.0), r2), &sphi, &cphi);
 
-    real pax = ma * ua.x, pay = ma * ua.y, paz = ma * ua.z;
-    real Ea = ma * ga, Eb = mb * gb, E = Ea + Eb;
-    const real iE = RF(1.0) / E;
-    real bx = (pax + mb * ub.x) * iE, by = (pay + mb * ub.y) * iE, bz = (paz + mb * ub.z) * iE;
-    real b2 = bx * bx + by * by + bz * bz;
-    real gc = r_rsqrt(RF(1.0) - b2);
-    real h = gc * gc / (gc + RF(1.0));
-    real bp = bx * pax + by * pay + bz * paz;
-    real c1 = h * bp - gc * Ea;
-    real sx = pax + c1 * bx, sy = pay + c1 * by, sz = paz + c1 * bz;
-    real p = r_sqrt(sx * sx + sy * sy + sz * sz);
-    if (p == RF(0.0)) return false;
+    const real pax = r_mul(ma, ua.x), pay = r_mul(ma, ua.y), paz = r_mul(ma, ua.z);
+    const real Ea = r_mul(ma, ga), iE = RF(1.0) / r_fma(mb, gb, Ea);
+    const real bx = r_mul(r_fma(mb, ub.x, pax), iE), by = r_mul(r_fma(mb, ub.y, pay), iE),
+               bz = r_mul(r_fma(mb, ub.z, paz), iE);
+    const real b2 = dot3(bx, by, bz, bx, by, bz);
+    const real gc = r_rsqrt(r_add(RF(1.0), -b2));
+    const real h = r_mul(gc, gc) / r_add(gc, RF(1.0));
+    const real bp = dot3(bx, by, bz, pax, pay, paz);
+    const real c1 = r_fma(h, bp, -r_mul(gc, Ea));
+    const real sx = r_fma(c1, bx, pax), sy = r_fma(c1, by, pay), sz = r_fma(c1, bz, paz);
+    const real p = r_sqrt(dot3(sx, sy, sz, sx, sy, sz));
+    if (p == RF(0.0)) return Collided{ua, ub, 0};
     const real ip = RF(1.0) / p;
-    real nx = sx * ip, ny = sy * ip, nz = sz * ip;
-    real d2 = delta * delta;
-    const real id2 = RF(1.0) / (RF(1.0) + d2);
-    real st = RF(2.0) * delta * id2, ct = (RF(1.0) - d2) * id2;
+    const real nx = r_mul(sx, ip), ny = r_mul(sy, ip), nz = r_mul(sz, ip);
+    const real id2 = RF(1.0) / r_fma(delta, delta, RF(1.0));
+    const real st = r_mul(r_mul(RF(2.0), delta), id2), ct = r_mul(r_fma(-delta, delta, RF(1.0)), id2);
     // azimuth frame (e1, e2) about n: on the z axis while n is at least 30
     // degrees from it, on the x axis otherwise (no division by a small
     // component, so FP32 rounding is not amplified near the poles)
     real e1x, e1y, e1z, e2x, e2y, e2z;
-    const real np2 = nx * nx + ny * ny;
+    const real np2 = r_fma(nx, nx, r_mul(ny, ny));
     if (np2 >= RF(0.25)) {
         const real np = r_sqrt(np2), inp = RF(1.0) / np;
-        e1x = nx * nz * inp; e1y = ny * nz * inp; e1z = -np;
-        e2x = -ny * inp; e2y = nx * inp; e2z = RF(0.0);
+        e1x = r_mul(r_mul(nx, nz), inp); e1y = r_mul(r_mul(ny, nz), inp); e1z = -np;
+        e2x = r_mul(-ny, inp); e2y = r_mul(nx, inp); e2z = RF(0.0);
     } else {
-        const real nq = r_sqrt(ny * ny + nz * nz), inq = RF(1.0) / nq;
-        e2x = RF(0.0); e2y = nz * inq; e2z = -ny * inq;
-        e1x = nq; e1y = -nx * ny * inq; e1z = -nx * nz * inq;
+        const real nq = r_sqrt(r_fma(nz, nz, r_mul(ny, ny))), inq = RF(1.0) / nq;
+        e2x = RF(0.0); e2y = r_mul(nz, inq); e2z = r_mul(-ny, inq);
+        e1x = nq; e1y = r_mul(r_mul(-nx, ny), inq); e1z = r_mul(r_mul(-nx, nz), inq);
     }
-    real qx = p * (ct * nx + st * cphi * e1x + st * sphi * e2x);
-    real qy = p * (ct * ny + st * cphi * e1y + st * sphi * e2y);
-    real qz = p * (ct * nz + st * cphi * e1z + st * sphi * e2z);
-    real Eas = r_sqrt(ma * ma + p * p), Ebs = r_sqrt(mb * mb + p * p);
-    real bq = bx * qx + by * qy + bz * qz;
-    real ca = h * bq + gc * Eas, cb = -h * bq + gc * Ebs;
-    real wm = wa > wb ? wa : wb;
+    const real sc = r_mul(st, cphi), ss = r_mul(st, sphi);
+    const real qx = r_mul(p, r_fma(ss, e2x, r_fma(ct, nx, r_mul(sc, e1x))));
+    const real qy = r_mul(p, r_fma(ss, e2y, r_fma(ct, ny, r_mul(sc, e1y))));
+    const real qz = r_mul(p, r_fma(ss, e2z, r_fma(ct, nz, r_mul(sc, e1z))));
+    const real pp = r_mul(p, p);
+    const real Eas = r_sqrt(r_fma(ma, ma, pp)), Ebs = r_sqrt(r_fma(mb, mb, pp));
+    const real bq = dot3(bx, by, bz, qx, qy, qz);
+    const real hb = r_mul(h, bq);
+    const real ca = r_fma(gc, Eas, hb), cb = r_fma(gc, Ebs, -hb);
+    const real wm = wa > wb ? wa : wb;
     if (r3 < wb / wm) {
         const real ima = RF(1.0) / ma;
-        ua.x = (qx + ca * bx) * ima; ua.y = (qy + ca * by) * ima; ua.z = (qz + ca * bz) * ima;
+        ua.x = r_mul(r_fma(ca, bx, qx), ima); ua.y = r_mul(r_fma(ca, by, qy), ima); ua.z = r_mul(r_fma(ca, bz, qz), ima);
     }
     if (r3 < wa / wm) {
         const real imb = RF(1.0) / mb;
-        ub.x = (-qx + cb * bx) * imb; ub.y = (-qy + cb * by) * imb; ub.z = (-qz + cb * bz) * imb;
+        ub.x = r_mul(r_fma(cb, bx, -qx), imb); ub.y = r_mul(r_fma(cb, by, -qy), imb);
+        ub.z = r_mul(r_fma(cb, bz, -qz), imb);
     }
-    return true;
+    return Collided{ua, ub, 1};
 }
 
 // relativistic Boris: q/m in e/m_e, dt fs, normalized fields

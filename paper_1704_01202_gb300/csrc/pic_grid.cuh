@@ -427,24 +427,17 @@ __global__ void k_photon_energy(const ph2 *ph, int ncell, int nb, const real *hv
     if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(out, v);
 }
 
-// the in-cell ordering of one cell (the cell kernel's warp_sort of the
-// kernel instance RMAX), run by one warp on given keys and ids:
-// order[k] = slot at position k
-template <int RMAX>
-__global__ void k_order_check(const unsigned long long *key_in, const unsigned long long *id_in, int n,
-                              unsigned short *order)
+// the in-cell ordering of one cell as the cell kernel forms it (RMAX up to
+// 512: one warp; TW warps above), run on given keys and ids: order[k] =
+// index of the entry at position k
+template <int RMAX, int TW>
+__global__ void __launch_bounds__(32 * TW) k_order_check(const unsigned long long *key_in, const unsigned long long *id_in,
+                                                         int n, unsigned short *order)
 {
-    extern __shared__ __align__(16) char sm[];
-    unsigned long long *key = (unsigned long long *)sm;                  // [n]
-    unsigned long long *id = key + n;                                     // [n]
-    unsigned long long *buf = id + n;                                     // [2 n]
-    int *hist = (int *)(buf + 2 * n);                                     // [256]
-    unsigned short *slot = (unsigned short *)(hist + 256);               // [n]
-    const int lane = threadIdx.x;
-    for (int k = lane; k < n; k += 32) { key[k] = key_in[k]; id[k] = id_in[k]; slot[k] = (unsigned short)k; }
-    __syncwarp();
-    warp_sort<unsigned long long, RMAX>(key, id, slot, key, buf, hist, n, lane);
-    for (int k = lane; k < n; k += 32) order[k] = slot[k];
+    extern __shared__ unsigned words[];                                   // [2 n]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned mask = order_cell<RMAX, TW>(GivenKeys{key_in, id_in}, words, words + n, n, warp, lane);
+    for (int k = threadIdx.x; k < n; k += 32 * TW) order[k] = (unsigned short)(words[k] & mask);
 }
 
 // ---------------- initial plasma on the device ----------------
