@@ -601,9 +601,16 @@ pic_status launch_step(pic_ctx *c)
     pa.ncell = c->ncell; pa.cell_slab = c->cell_slab; pa.slabs = c->d_slab; pa.tally = c->d_tally;
     pa.fldE = c->E[c->ecur]; pa.fldB = c->B; pa.npts = c->npts; pa.J = c->J;
     pa.err = c->counters + CNT_ERR; pa.work = c->counters + CNT_WORK_PUSH;
-    k_push<<<c->grid_push, 32 * PUSH_WARPS, 0, st>>>(pa);
-    k_push_new<<<c->nsm * 2, 256, 0, st>>>(pa);
-    c->launches += 2;
+    const bool d2 = c->slabs[0].ny > 1;
+    // fewer cells than the warps that fill the SMs (16 each, the cell
+    // kernel's residency): a team of warps per cell.  Measured per step, one
+    // warp | team: 700 cells 60 | 33 us, 4096 (2D) 52 | 52, 6000 39 | 44,
+    // 13000 129 | 174.
+    if (c->ncell < 16 * c->nsm)
+        (d2 ? k_push_team<2, PUSH_TEAM> : k_push_team<1, PUSH_TEAM>)<<<c->ncell + PUSH_NEW_CTAS, 32 * PUSH_TEAM, 0, st>>>(pa);
+    else
+        (d2 ? k_push<2> : k_push<1>)<<<c->grid_push, 32 * PUSH_WARPS, 0, st>>>(pa);
+    ++c->launches;
     CK(cudaGetLastError());
     if (ev) CK(cudaEventRecord(ev[3], st));
     const int nxt = c->cur ^ 1;
@@ -887,7 +894,7 @@ pic_status ctx_create(pic_ctx **out, int nslot, int slot_cells, int slot_pts, in
         if ((rc = configure_cell_launch(c, he, hi, 100, 25)) != PIC_OK) { pic_free(c); return rc; }
     }
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_push, 32 * PUSH_WARPS, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, slot_rows > 1 ? k_push<2> : k_push<1>, 32 * PUSH_WARPS, 0);
     if (e != cudaSuccess) { rc = cuda_fail(c, e, "push occupancy"); pic_free(c); return rc; }
     c->grid_push = std::max(1, occ) * c->nsm;
     *out = c;

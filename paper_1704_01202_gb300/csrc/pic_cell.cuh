@@ -424,40 +424,12 @@ __device__ inline CellMem carve(char *base, int ce, int ci, NewE *nw)
     return m;
 }
 
-// ---------------------------------------------------------------------
-// field gather (CIC from the staggered Yee grid; zero outside [0, nx])
-// ---------------------------------------------------------------------
+// grid of one slab, as the deposit of long moves takes it
 struct SlabGrid {
     int nx, ny, W;       // W = nx + 1 points per row
-    const real *fe;     // ex of this slab (ey, ez follow with stride npts)
-    const real *fb;     // bx of this slab
     int npts;            // stride between components
     int fo;              // first grid point of the slab
 };
-
-__device__ __forceinline__ real grid_interp(const real *F, const SlabGrid &g, int cx, int cy,
-                                             real xi, real eta, bool hx, bool hy)
-{
-    real xs = xi - (hx ? RF(0.5) : RF(0.0)), ys = eta - (hy ? RF(0.5) : RF(0.0));
-    int ax = (int)r_floor(xs), ay = (int)r_floor(ys);
-    real fx = xs - (real)ax, fy = ys - (real)ay;
-    int imax = hx ? g.nx - 1 : g.nx;
-    real v = RF(0.0);
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-        int i = cx + ax + a;
-        if (i < 0 || i > imax) continue;
-        real wx = a ? fx : RF(1.0) - fx;
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            int j = cy + ay + b;
-            j %= g.ny; if (j < 0) j += g.ny;
-            real wy = b ? fy : RF(1.0) - fy;
-            v += wx * wy * __ldg(F + (size_t)j * g.W + i);
-        }
-    }
-    return v;
-}
 
 // ---------------------------------------------------------------------
 // current deposit
@@ -581,51 +553,6 @@ __device__ __noinline__ void deposit_long(const SlabGrid &g, unsigned long long 
             }
         }
     }
-}
-
-// ---------------------------------------------------------------------
-// push of one particle: gather, Boris, move, deposit; returns the next
-// cell (local index) or -1 when it left through an x boundary
-// ---------------------------------------------------------------------
-template <int DIM, class Acc>
-__device__ __forceinline__ int push_one(const SlabDev &S, const SlabGrid &g, unsigned long long *J, int npts,
-                                        int cx, int cy, real &xi, real &eta, real &ux, real &uy, real &uz,
-                                        real qm, real qw, bool do_push, bool do_dep, Acc &A)
-{
-    if (!do_push) return cy * S.nx + cx;
-    real ex = grid_interp(g.fe, g, cx, cy, xi, eta, true, false);
-    real ey = grid_interp(g.fe + g.npts, g, cx, cy, xi, eta, false, true);
-    real ez = grid_interp(g.fe + 2 * g.npts, g, cx, cy, xi, eta, false, false);
-    real bx = grid_interp(g.fb, g, cx, cy, xi, eta, false, true);
-    real by = grid_interp(g.fb + g.npts, g, cx, cy, xi, eta, true, false);
-    real bz = grid_interp(g.fb + 2 * g.npts, g, cx, cy, xi, eta, true, true);
-    boris(ux, uy, uz, ex, ey, ez, bx, by, bz, qm, S.dt);
-    real ig = r_rsqrt(RF(1.0) + ux * ux + uy * uy + uz * uz);
-    real bxv = ux * ig, byv = uy * ig, bzv = uz * ig;
-    const real c = (real)kCnmPerFs;
-    real xn = xi + bxv * c * S.dt / S.dx;
-    real yn = DIM == 2 ? eta + byv * c * S.dt / S.dy : eta;
-    if (!(r_fabs(xn - xi) < RF(64.0) && r_fabs(yn - eta) < RF(64.0))) return -2;   // not finite: dropped
-    if (do_dep) {
-        if (r_fabs(xn - xi) < RF(1.0) && r_fabs(yn - eta) < RF(1.0)) {
-            if constexpr (DIM == 2) esirkepov2(xi, eta, xn, yn, qw, qw * bzv, RF(1.0), A);
-            else esirkepov1(xi, xn, qw, qw * byv, qw * bzv, RF(1.0), A);
-        } else {
-            deposit_long(g, J, npts, g.fo, cx, cy, xi, eta, xn, yn, qw, qw * byv, qw * bzv);
-        }
-    }
-    real fx = r_floor(xn), fy = r_floor(yn);
-    int ncx = cx + (int)fx;
-    int ncy = cy + (int)fy;
-    xi = xn - fx;
-    eta = yn - fy;
-    const real below1 = kBelow1;
-    if (xi >= RF(1.0)) xi = below1;
-    if (eta >= RF(1.0)) eta = below1;
-    if (DIM == 1) { ncy = 0; }
-    else { ncy %= S.ny; if (ncy < 0) ncy += S.ny; }
-    if (ncx < 0 || ncx >= S.nx) return -1;
-    return ncy * S.nx + ncx;
 }
 
 }  // namespace pic

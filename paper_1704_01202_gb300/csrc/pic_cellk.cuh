@@ -1141,13 +1141,14 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 32 * TW, TW == 1 ? 2 : 4) k_ce
     extern __shared__ __align__(kSmAlign) char smem[];
     __shared__ Tables T;
     __shared__ int round_base;
+    const int total = a.list ? *a.n_list : a.ncell;
+    if (total == 0) return;              // a tier no cell needs
     for (int k = threadIdx.x; k < (int)(sizeof(Tables) / sizeof(real)); k += blockDim.x)
         ((real *)&T)[k] = ((const real *)a.tab)[k];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nteam = TW == 1 ? blockDim.x >> 5 : 1;
     const int team = TW == 1 ? warp : 0;
     CellMem m = carve(smem + (size_t)team * cell_mem_bytes(a.cap_ce, a.cap_ci), a.cap_ce, a.cap_ci,
                       a.nw + ((size_t)blockIdx.x * nteam + team) * a.cap_new);
-    const int total = a.list ? *a.n_list : a.ncell;
     WarpTally wt;
     LaneTally lt{0, 0, 0, 0};
     wt.slab = -1;

@@ -540,15 +540,16 @@ __device__ __forceinline__ Collided binary_collision(real4 ua, real4 ub, real ma
 __device__ __forceinline__ void boris(real &ux, real &uy, real &uz, real ex, real ey, real ez,
                                       real bx, real by, real bz, real qm, real dt)
 {
-    real h = RF(0.5) * qm * dt;
-    real mx = ux + h * ex, my = uy + h * ey, mz = uz + h * ez;
-    real ig = r_rsqrt(RF(1.0) + mx * mx + my * my + mz * mz);
-    real tx = h * bx * ig, ty = h * by * ig, tz = h * bz * ig;
-    real t2 = tx * tx + ty * ty + tz * tz;
-    real s = RF(2.0) / (RF(1.0) + t2);
-    real px = mx + my * tz - mz * ty, py = my + mz * tx - mx * tz, pz = mz + mx * ty - my * tx;
-    real qx = mx + (py * tz - pz * ty) * s, qy = my + (pz * tx - px * tz) * s, qz = mz + (px * ty - py * tx) * s;
-    ux = qx + h * ex; uy = qy + h * ey; uz = qz + h * ez;
+    const real h = r_mul(r_mul(RF(0.5), qm), dt);
+    const real mx = r_fma(h, ex, ux), my = r_fma(h, ey, uy), mz = r_fma(h, ez, uz);
+    const real ig = r_rsqrt(r_fma(mz, mz, r_fma(my, my, r_fma(mx, mx, RF(1.0)))));
+    const real tx = r_mul(r_mul(h, bx), ig), ty = r_mul(r_mul(h, by), ig), tz = r_mul(r_mul(h, bz), ig);
+    const real s = RF(2.0) / r_add(RF(1.0), square3(tx, ty, tz));
+    const real px = r_fma(-mz, ty, r_fma(my, tz, mx)), py = r_fma(-mx, tz, r_fma(mz, tx, my)),
+               pz = r_fma(-my, tx, r_fma(mx, ty, mz));
+    const real qx = r_fma(r_fma(py, tz, -r_mul(pz, ty)), s, mx), qy = r_fma(r_fma(pz, tx, -r_mul(px, tz)), s, my),
+               qz = r_fma(r_fma(px, ty, -r_mul(py, tx)), s, mz);
+    ux = r_fma(h, ex, qx); uy = r_fma(h, ey, qy); uz = r_fma(h, ez, qz);
 }
 
 // isotropic momentum of kinetic energy ke (eV) for an electron

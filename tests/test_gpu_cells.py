@@ -55,3 +55,30 @@ def test_cell_sizes_one_step(tables, ppc_e, ppc_i):
     st = _busy(cfg, seed=4)
     g, o = _run_both(cfg, tables, st, 1, pulse=pl, photons=P.photons_uniform(cfg, pl, 0.5))
     _assert_parity(cfg, st, g, o)
+
+
+@pytest.mark.parametrize("ppc_e,ppc_i,T_e", [(31, 1, 10.0), (33, 32, 2e4), (100, 25, 3e5), (600, 130, 50.0)])
+def test_push_team_and_warp_agree(tables, ppc_e, ppc_i, T_e):
+    """A slab alone has fewer cells than fill the GPU (a block per cell in the
+    push); in a context of 4096 cells the same slab is pushed one warp per
+    cell.  Same state bit for bit, with created electrons, particles leaving
+    through the boundaries and moves of more than a cell (T_e = 3e5)."""
+    cfg = P.cfg_small_1d(nx=24, ppc_e=ppc_e, ppc_i=ppc_i, T_e_eV=T_e, flags=P.F_ALL, rad_every=1)
+    pl = P.Pulse(I_peak_Wcm2=3e17, fwhm_fs=30.0, t_peak_fs=0.0, hv_eV=1700.0, n_bins=2, bandwidth_eV=60.0)
+    st = _busy(cfg, seed=6)
+    ce, ci = pkg.default_capacity(st.n_e, st.n_i, cfg.Z_init)
+    one = pkg.Slab(cfg, tables, pl)
+    one.load(st)
+    many = pkg.Batch(tables, 2, 2048, 2 * ce, 2 * ci)
+    slot = many.admit(cfg, st, pl)
+    one.step(5)
+    many.step(5)
+    for a, b in ((one.electrons(), many.electrons(slot)), (one.ions(), many.ions(slot))):
+        ka, kb = np.argsort(a["id"]), np.argsort(b["id"])
+        for q in a:
+            assert np.array_equal(a[q][ka], b[q][kb]), q
+    da, db = one.diagnostics(), many.diagnostics(slot)
+    assert da["counts"] == db["counts"]
+    assert ppc_e != 100 or da["counts"]["ESC_E"] > 0
+    one.close()
+    many.close()
