@@ -33,9 +33,11 @@ namespace {
 
 // device counters; [0, CNT_STEP_ZERO) are cleared at the start of a step
 constexpr int CNT_APPEND = 0, CNT_WORK = 1, CNT_WORK_T1 = 2, CNT_WORK_BIG = 3, CNT_OVF = 4, CNT_OVF2 = 5,
-              CNT_WORK_PUSH = 6, CNT_WORK_T2 = 7, CNT_OVF3 = 8, CNT_STEP_ZERO = 9, CNT_ERR = 10, CNT_MAXE = 11,
-              CNT_MAXI = 12, CNT_NLOAD = 13, CNT_HIST_E = 16, CNT_HIST_I = CNT_HIST_E + NHIST,
+              CNT_WORK_PUSH = 6, CNT_WORK_T2 = 7, CNT_OVF3 = 8, CNT_STEP_ZERO = 9, CNT_ERR = 10, CNT_NLOAD = 11,
+              CNT_MAXE = 12, CNT_MAXI = 13, CNT_HIST_E = 16, CNT_HIST_I = CNT_HIST_E + NHIST,
               NCOUNTERS = CNT_HIST_I + NHIST;
+// (k_begin clears [0, CNT_STEP_ZERO) and [CNT_MAXE, NCOUNTERS), 16-byte aligned)
+static_assert(CNT_MAXE % 4 == 0, "alignment of the cleared counters");
 constexpr int NEV = 6;   // timing events per step
 // largest cell of the one-warp pass (the FP64 build's staging is twice as
 // wide and takes half the populations into the same shared memory)
@@ -440,7 +442,9 @@ CellArgs cell_args(pic_ctx *c, CellTier tier)
     return a;
 }
 
-pic_status run_scan(pic_ctx *c, int species_mask, int dst)
+// cell starts csE / csI[dst] from the counts; zeroed: the histograms are
+// zero already (k_begin)
+pic_status run_scan(pic_ctx *c, int species_mask, int dst, bool zeroed = false)
 {
     ScanArgs s{};
     int k = 0;
@@ -452,17 +456,21 @@ pic_status run_scan(pic_ctx *c, int species_mask, int dst)
         s.cnt[k] = c->cnt_i; s.cs[k] = c->csI[dst]; s.bsum[k] = c->bsum_i;
         s.maxc[k] = c->counters + CNT_MAXI; s.hist[k] = c->counters + CNT_HIST_I; ++k;
     }
-    for (int q = 0; q < k; ++q) {
+    for (int q = 0; q < k && !zeroed; ++q) {
         CK(cudaMemsetAsync(s.maxc[q], 0, sizeof(int), c->stream));
         CK(cudaMemsetAsync(s.hist[q], 0, sizeof(int) * NHIST, c->stream));
     }
     s.n = c->ncell;
     s.nblk = c->nblk;
     dim3 g1(c->nblk, k);
-    k_scan_reduce<<<g1, SCAN_T, 0, c->stream>>>(s);
-    k_scan_blocks<<<dim3(1, k), SCAN_T, 0, c->stream>>>(s);
-    k_scan_final<<<g1, SCAN_T, 0, c->stream>>>(s);
-    c->launches += 3;
+    if (c->nblk <= SCAN_SELF) {
+        k_scan_final<true><<<g1, SCAN_T, 0, c->stream>>>(s);
+    } else {
+        k_scan_reduce<<<g1, SCAN_T, 0, c->stream>>>(s);
+        k_scan_final<false><<<g1, SCAN_T, 0, c->stream>>>(s);
+        ++c->launches;
+    }
+    ++c->launches;
     CK(cudaGetLastError());
     return PIC_OK;
 }
@@ -545,9 +553,21 @@ pic_status launch_step(pic_ctx *c)
     const pic_ctx::StepShape shape = step_shape(c);
     cudaEvent_t *ev = timing_slot(c);
     if (ev) CK(cudaEventRecord(ev[0], st));
-    CK(cudaMemsetAsync(c->cnt_e, 0, sizeof(int) * 4 * (size_t)c->ncell, st));   // cnt_e cnt_i fill_e fill_i
-    CK(cudaMemsetAsync(c->counters, 0, sizeof(int) * CNT_STEP_ZERO, st));          // append, work counters, lists
-    CK(cudaMemsetAsync(c->J, 0, sizeof(unsigned long long) * 3 * (size_t)c->npts, st));
+    {
+        nv.phase(shape.march ? "photon march" : "step begin");
+        BeginArgs b{};
+        b.m = MarchArgs{c->d_slab, c->d_steps, c->row_slab, c->row_idx, c->photons, c->d_tally};
+        b.march_blocks = shape.march ? c->nrows : 0;
+        auto zero = [&](int q, void *p, size_t bytes) { b.z[q] = (uint4 *)p; b.nz[q] = (long long)bytes; };
+        zero(0, c->cnt_e, sizeof(int) * 4 * (size_t)c->ncell);            // cnt_e cnt_i fill_e fill_i
+        zero(1, c->J, sizeof(unsigned long long) * 3 * (size_t)c->npts);
+        zero(2, c->counters, sizeof(int) * CNT_STEP_ZERO);                // append, work counters, lists
+        zero(3, c->counters + CNT_MAXE, sizeof(int) * (NCOUNTERS - CNT_MAXE));   // largest cells, histograms
+        const size_t words = 4 * (size_t)c->ncell + 6 * (size_t)c->npts;
+        const int zb = (int)std::min<size_t>((size_t)c->nsm * 8, words / (4 * 256) + 1);
+        k_begin<<<b.march_blocks + zb, 256, shape.march ? (size_t)c->max_row_nx * 8 : 0, st>>>(b);
+        ++c->launches;
+    }
     if (shape.rt) {
         nv.phase("radiation transport");
         // radiation transport (single-slab contexts): the kernels return at
@@ -565,11 +585,6 @@ pic_status launch_step(pic_ctx *c)
             ++c->launches;
         }
         k_rt_publish<<<std::min((S.ncell + 255) / 256, c->nsm * 8), 256, 0, st>>>(ra);
-        ++c->launches;
-    } else if (shape.march) {
-        nv.phase("photon march");
-        MarchArgs m{c->d_slab, c->d_steps, c->row_slab, c->row_idx, c->photons, c->d_tally};
-        k_march<<<c->nrows, 256, (size_t)c->max_row_nx * 8, st>>>(m);
         ++c->launches;
     }
     if (ev) CK(cudaEventRecord(ev[1], st));
@@ -615,16 +630,15 @@ pic_status launch_step(pic_ctx *c)
     if (ev) CK(cudaEventRecord(ev[3], st));
     const int nxt = c->cur ^ 1;
     nv.phase("counting sort");
-    pic_status r = run_scan(c, 3, nxt);
+    pic_status r = run_scan(c, 3, nxt, true);
     if (r != PIC_OK) return r;
     int sgrid = c->nsm * 8;
     ScatterArgs se{c->eA0, c->eA1, c->ekey, c->csE[c->cur] + c->ncell, c->counters + CNT_APPEND,
                    c->csE[nxt], c->fill_e, c->eB0, c->eB1, c->cap_e};
-    k_scatter<<<sgrid, 256, 0, st>>>(se);
     ScatterArgs si{c->iA0, c->iA1, c->ikey, c->csI[c->cur] + c->ncell, nullptr, c->csI[nxt], c->fill_i, c->iB0, c->iB1,
                    c->cap_i};
-    k_scatter<<<sgrid, 256, 0, st>>>(si);
-    c->launches += 2;
+    k_scatter<<<sgrid, 256, 0, st>>>(se, si);
+    ++c->launches;
     if (ev) CK(cudaEventRecord(ev[4], st));
     if (shape.field) {
         nv.phase("fields");
@@ -643,7 +657,8 @@ pic_status launch_step(pic_ctx *c)
             c->launches += 3;
         }
     }
-    k_advance<<<(c->nslot + 127) / 128, 128, 0, st>>>(c->d_steps, c->d_slab, c->nslot, c->slab_app, c->slab_err);
+    const AdvanceArgs adv{c->d_steps, c->d_slab, c->nslot, c->slab_app, c->slab_err};
+    k_advance<<<(c->nslot + 127) / 128, 128, 0, st>>>(adv);
     ++c->launches;
     CK(cudaGetLastError());
     if (ev) CK(cudaEventRecord(ev[5], st));
@@ -887,8 +902,8 @@ pic_status ctx_create(pic_ctx **out, int nslot, int slot_cells, int slot_pts, in
     if (e != cudaSuccess) { rc = cuda_fail(c, e, "init copies"); pic_free(c); return rc; }
     c->smem_big = cell_mem_bytes(BIG_CE, BIG_CI);
     c->grid_big = cell_grid(c, 1, TEAM, BIG_CE, BIG_CI);
-    e = cudaFuncSetAttribute(k_march, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * 8);
-    if (e != cudaSuccess) { rc = cuda_fail(c, e, "march attribute"); pic_free(c); return rc; }
+    e = cudaFuncSetAttribute(k_begin, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * 8);
+    if (e != cudaSuccess) { rc = cuda_fail(c, e, "begin attribute"); pic_free(c); return rc; }
     {
         int he[NHIST] = {}, hi[NHIST] = {};
         if ((rc = configure_cell_launch(c, he, hi, 100, 25)) != PIC_OK) { pic_free(c); return rc; }
@@ -973,7 +988,7 @@ pic_status sort_species(pic_ctx *c, bool electrons, int64_t n)
     if (r != PIC_OK) return r;
     ScatterArgs sa{s0, s1, k, c->counters + CNT_NLOAD, nullptr, electrons ? c->csE[c->cur] : c->csI[c->cur], fill, d0, d1,
                    electrons ? c->cap_e : c->cap_i};
-    k_scatter<<<c->nsm * 4, 256, 0, st>>>(sa);
+    k_scatter<<<c->nsm * 8, 256, 0, st>>>(sa, ScatterArgs{});
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(st));
     return PIC_OK;
@@ -1029,7 +1044,7 @@ pic_status resort_with(pic_ctx *c, const std::vector<real4> &e0, const std::vect
         if (r != PIC_OK) return r;
         ScatterArgs sa{A0, A1, key, c->counters + CNT_NLOAD, nullptr, el ? c->csE[nxt] : c->csI[nxt], fill, B0, B1,
                        el ? c->cap_e : c->cap_i};
-        k_scatter<<<c->nsm * 4, 256, 0, st>>>(sa);
+        k_scatter<<<c->nsm * 8, 256, 0, st>>>(sa, ScatterArgs{});
         CK(cudaGetLastError());
         CK(cudaStreamSynchronize(st));     // tot is read by the device; the next species reuses it
     }
