@@ -281,8 +281,9 @@ size_t pic_checkpoint_bytes(pic_ctx *c);
 pic_status pic_checkpoint(pic_ctx *c, void *host, size_t bytes);
 pic_status pic_restore(pic_ctx *c, const void *host, size_t bytes);
 
-/* Advance n PIC steps (asynchronous on the context stream; the call
- * synchronizes every 32 steps to re-size the cell tiers).  Device-side
+/* Advance n PIC steps (asynchronous on the context stream; with more than
+ * a few hundred cells the call synchronizes every 32 steps to re-size the
+ * cell tiers).  Device-side
  * problems are latched and reported by the next synchronizing call:
  * PIC_ERR_CAPACITY when the electrons created in a step would exceed the
  * context's capacity (or a cell outgrows the large-cell pass) and

@@ -108,6 +108,8 @@ struct pic_ctx {
     int t1_ce = 0, t1_ci = 0, t1_wpc = 1;    // t1_ce == 0: no tier 1
     int t2_ce = 0, t2_ci = 0, t2_wpc = 1;    // t2_ce == 0: no tier 2
     size_t smem_main = 0, smem_t1 = 0, smem_t2 = 0, smem_big = 0;
+    bool teams = false;                  // few cells: a team of warps takes each (team_warps)
+    bool whole = false;                  // fewer still: tier 0 stages the largest cells itself
     int nsm = 0, grid_main = 0, grid_t1 = 0, grid_t2 = 0, grid_big = 0, grid_push = 0;
     NewE *nw = nullptr;                  // created-electron scratch of the cell launches
     size_t nw_entries = 0;
@@ -183,10 +185,15 @@ T *carve_arena(pic_ctx *c, size_t count)
 // 1536 take one warp a CTA) for every warp resident at once, at most 16 a
 // SM (the register-bound instances) on up to 192 SMs, and no more warps
 // than cells (plus a CTA).  Launch grids are clamped to the slices.
+// Contexts of up to WHOLE_CELLS cells (and two an SM: that staging is 100 KB)
+// stage every cell at the large-cell pass's size: no pass for what outgrows
+// its tier, and nothing to re-size between steps.  257 cells of 123 electrons
+// and 31 ions, a step: 94 -> 57 us with the one-launch field update.
+constexpr int WHOLE_CELLS = 384;
 size_t nw_scratch_entries(int ncell)
 {
     const size_t warps = std::min<size_t>(192 * 16, (size_t)ncell + 64);
-    return warps * 768;
+    return warps * (ncell <= WHOLE_CELLS ? 3 * BIG_CI : 768);
 }
 
 size_t arena_need(int ncell, int npts, int nblk, int cap_e, int cap_i, int nslot, int nrows)
@@ -224,35 +231,40 @@ double sigma_table(const pic_ctx *c, int s, double hv)
     return std::exp(std::log(v[lo]) + f * std::log(v[lo + 1] / v[lo]));
 }
 
-// Warps per cell of a launch staging up to ce electrons and ci ions: one
+// Warps per cell of a launch staging up to ce electrons and ci ions.  One
 // warp sorts up to 512 entries in registers; larger cells take a block of
 // TEAM warps, which share the staging (a 1024-electron cell's is ~50 KB: at
-// one warp a cell, 8 warps an SM): 700 cells of ~820 electrons and 102 ions,
-// 217 us a step at one warp a cell, 136 us at four.
+// one warp a cell, 8 warps an SM).  So do all cells of a context so small
+// that each can have a team at once (16 warps an SM): what counts there is the
+// time of one cell.  Measured per step, one warp | four (cell kernel): 700
+// cells of 820 electrons and 102 ions 217 | 136 us (the split at 512), 128 of
+// 256 + 64 75 | 51, 257 of 123 + 31 91 | 71, 64 of 26 + 6 36 | 34; beyond,
+// 4096 of 80 + 20 75 | 151, 6000 of 64 + 16 119 | 295.  Eight warps: the same
+// on the smallest, slower from 700 cells on (157 us).
 constexpr int TEAM = 4;
-int team_warps(int ce, int ci) { return std::max(ce, ci) > 512 ? TEAM : 1; }
+int team_warps(const pic_ctx *c, int ce, int ci) { return c->teams || std::max(ce, ci) > 512 ? TEAM : 1; }
 
 // the cell-kernel instance of such a launch
 typedef void (*CellKernel)(CellArgs);
-CellKernel cell_kernel(int ce, int ci)
+CellKernel cell_kernel(const pic_ctx *c, int ce, int ci)
 {
-    if (team_warps(ce, ci) > 1) return k_cell<2048, TEAM>;
+    if (team_warps(c, ce, ci) > 1) return k_cell<2048, TEAM>;
     return std::max(ce, ci) <= 128 ? k_cell<128, 1> : k_cell<512, 1>;
 }
 
 // shared memory of a CTA of wpc warps (wpc / team_warps cells)
-size_t cell_smem(int ce, int ci, int wpc) { return cell_mem_bytes(ce, ci) * (wpc / team_warps(ce, ci)); }
+size_t cell_smem(const pic_ctx *c, int ce, int ci, int wpc) { return cell_mem_bytes(ce, ci) * (wpc / team_warps(c, ce, ci)); }
 
 // largest warps per CTA of the cell kernel whose staging fits 200 KB, at
 // most 8 and at most what the instance's launch bounds allow; a team is a
 // CTA
-int max_wpc(int ce, int ci)
+int max_wpc(const pic_ctx *c, int ce, int ci)
 {
-    if (team_warps(ce, ci) > 1) return team_warps(ce, ci);
+    if (team_warps(c, ce, ci) > 1) return team_warps(c, ce, ci);
     const size_t per = cell_mem_bytes(ce, ci);
     int lim = 8;
     cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, cell_kernel(ce, ci)) == cudaSuccess && fa.maxThreadsPerBlock >= 32)
+    if (cudaFuncGetAttributes(&fa, cell_kernel(c, ce, ci)) == cudaSuccess && fa.maxThreadsPerBlock >= 32)
         lim = std::min(lim, fa.maxThreadsPerBlock / 32);
     return std::max(1, (int)std::min<size_t>(lim, (200 * 1024) / per));
 }
@@ -261,7 +273,7 @@ int max_wpc(int ce, int ci)
 // every SM, as many as the global scratch has team slices for
 int cell_grid(const pic_ctx *c, int occ, int wpc, int ce, int ci)
 {
-    const size_t cap = c->nw_entries / ((size_t)(wpc / team_warps(ce, ci)) * 3 * ci);
+    const size_t cap = c->nw_entries / ((size_t)(wpc / team_warps(c, ce, ci)) * 3 * ci);
     return std::max(1, (int)std::min<size_t>((size_t)std::max(1, occ) * c->nsm, std::min<size_t>(cap, 1 << 30)));
 }
 
@@ -288,12 +300,12 @@ pic_status cell_smem_attr(pic_ctx *c)
 // go to the larger CTA.
 int best_wpc(pic_ctx *c, int ce, int ci)
 {
-    if (cell_smem_attr(c) != PIC_OK) return max_wpc(ce, ci);
-    if (team_warps(ce, ci) > 1) return team_warps(ce, ci);
+    if (cell_smem_attr(c) != PIC_OK) return max_wpc(c, ce, ci);
+    if (team_warps(c, ce, ci) > 1) return team_warps(c, ce, ci);
     int best = 1, best_warps = 0;
-    for (int w = 1; w <= max_wpc(ce, ci); ++w) {
+    for (int w = 1; w <= max_wpc(c, ce, ci); ++w) {
         int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(ce, ci), 32 * w, cell_smem(ce, ci, w)) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(c, ce, ci), 32 * w, cell_smem(c, ce, ci, w)) !=
             cudaSuccess)
             continue;
         if (occ * w >= best_warps) { best_warps = occ * w; best = w; }
@@ -305,11 +317,11 @@ int best_wpc(pic_ctx *c, int ce, int ci)
 pic_status set_wpc(pic_ctx *c, int wpc)
 {
     c->wpc = wpc;
-    c->smem_main = cell_smem(c->cap_ce, c->cap_ci, wpc);
+    c->smem_main = cell_smem(c, c->cap_ce, c->cap_ci, wpc);
     pic_status r = cell_smem_attr(c);
     if (r != PIC_OK) return r;
     int occ = 0;
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(c->cap_ce, c->cap_ci), wpc * 32, c->smem_main));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(c, c->cap_ce, c->cap_ci), wpc * 32, c->smem_main));
     c->grid_main = cell_grid(c, occ, wpc, c->cap_ce, c->cap_ci);
     return PIC_OK;
 }
@@ -345,6 +357,12 @@ int round_cap(int v, int q, int lo, int hi) { return std::min(hi, std::max(lo, (
 // that stay resident.
 pic_status configure_cell_launch(pic_ctx *c, const int *hist_e, const int *hist_i, int max_e, int max_i)
 {
+    if (c->whole) {
+        c->cap_ce = BIG_CE; c->cap_ci = BIG_CI; c->cap_new = 3 * BIG_CI;
+        c->t1_ce = c->t1_ci = c->t2_ce = c->t2_ci = 0;
+        c->smem_t1 = c->smem_t2 = 0;
+        return set_wpc(c, TEAM);
+    }
     // the largest cells x 1.25, kept well inside int (the tiers stop at 2048)
     const int want_e = (int)std::min(max_e * 1.25 + 1.0, (double)(1 << 30));
     const int want_i = (int)std::min(max_i * 1.25 + 1.0, (double)(1 << 30));
@@ -359,12 +377,12 @@ pic_status configure_cell_launch(pic_ctx *c, const int *hist_e, const int *hist_
         c->t1_ce = round_cap(want_e, 128, ce, 1024);
         c->t1_ci = round_cap(want_i, 32, ci, 256);
         c->t1_wpc = best_wpc(c, c->t1_ce, c->t1_ci);
-        c->smem_t1 = cell_smem(c->t1_ce, c->t1_ci, c->t1_wpc);
+        c->smem_t1 = cell_smem(c, c->t1_ce, c->t1_ci, c->t1_wpc);
         if (want_e > c->t1_ce || want_i > c->t1_ci) {
             c->t2_ce = round_cap(want_e, 256, c->t1_ce, BIG_CE);
             c->t2_ci = round_cap(want_i, 64, c->t1_ci, BIG_CI);
             c->t2_wpc = best_wpc(c, c->t2_ce, c->t2_ci);
-            c->smem_t2 = cell_smem(c->t2_ce, c->t2_ci, c->t2_wpc);
+            c->smem_t2 = cell_smem(c, c->t2_ce, c->t2_ci, c->t2_wpc);
         }
     }
     int wpc = best_wpc(c, ce, ci);
@@ -374,12 +392,12 @@ pic_status configure_cell_launch(pic_ctx *c, const int *hist_e, const int *hist_
     if (r != PIC_OK) return r;
     int occ = 0;
     if (c->t1_ce) {
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(c->t1_ce, c->t1_ci), c->t1_wpc * 32,
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(c, c->t1_ce, c->t1_ci), c->t1_wpc * 32,
                                                          c->smem_t1));
         c->grid_t1 = cell_grid(c, occ, c->t1_wpc, c->t1_ce, c->t1_ci);
     }
     if (c->t2_ce) {
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(c->t2_ce, c->t2_ci), c->t2_wpc * 32,
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cell_kernel(c, c->t2_ce, c->t2_ci), c->t2_wpc * 32,
                                                          c->smem_t2));
         c->grid_t2 = cell_grid(c, occ, c->t2_wpc, c->t2_ce, c->t2_ci);
     }
@@ -419,7 +437,7 @@ CellArgs cell_args(pic_ctx *c, CellTier tier)
     if (tier == TIER0) {
         a.work = c->counters + CNT_WORK;
         a.list = nullptr; a.n_list = nullptr;
-        a.ovf_list = c->ovf_list; a.ovf_count = c->counters + CNT_OVF;
+        a.ovf_list = c->whole ? nullptr : c->ovf_list; a.ovf_count = c->counters + CNT_OVF;
         a.cap_ce = c->cap_ce; a.cap_ci = c->cap_ci; a.cap_new = c->cap_new;
     } else if (tier == TIER1) {
         a.work = c->counters + CNT_WORK_T1;
@@ -591,20 +609,23 @@ pic_status launch_step(pic_ctx *c)
     if (c->cell_ev_on) CK(cudaEventRecord(c->cell_ev[0], st));
     nv.phase("collisions and atomic processes");
     CellArgs a0 = cell_args(c, TIER0);
-    cell_kernel(c->cap_ce, c->cap_ci)<<<c->grid_main, c->wpc * 32, c->smem_main, st>>>(a0);
+    cell_kernel(c, c->cap_ce, c->cap_ci)<<<c->grid_main, c->wpc * 32, c->smem_main, st>>>(a0);
     if (c->t1_ce) {
         CellArgs a1 = cell_args(c, TIER1);
-        cell_kernel(c->t1_ce, c->t1_ci)<<<c->grid_t1, c->t1_wpc * 32, c->smem_t1, st>>>(a1);
+        cell_kernel(c, c->t1_ce, c->t1_ci)<<<c->grid_t1, c->t1_wpc * 32, c->smem_t1, st>>>(a1);
         ++c->launches;
     }
     if (c->t2_ce) {
         CellArgs a2 = cell_args(c, TIER2);
-        cell_kernel(c->t2_ce, c->t2_ci)<<<c->grid_t2, c->t2_wpc * 32, c->smem_t2, st>>>(a2);
+        cell_kernel(c, c->t2_ce, c->t2_ci)<<<c->grid_t2, c->t2_wpc * 32, c->smem_t2, st>>>(a2);
         ++c->launches;
     }
-    CellArgs ab = cell_args(c, TIER_BIG);
-    cell_kernel(BIG_CE, BIG_CI)<<<c->grid_big, 32 * TEAM, c->smem_big, st>>>(ab);
-    c->launches += 2;
+    ++c->launches;
+    if (!c->whole) {
+        CellArgs ab = cell_args(c, TIER_BIG);
+        cell_kernel(c, BIG_CE, BIG_CI)<<<c->grid_big, 32 * TEAM, c->smem_big, st>>>(ab);
+        ++c->launches;
+    }
     if (c->cell_ev_on) CK(cudaEventRecord(c->cell_ev[1], st));
     CK(cudaGetLastError());
     if (ev) CK(cudaEventRecord(ev[2], st));
@@ -640,6 +661,7 @@ pic_status launch_step(pic_ctx *c)
     k_scatter<<<sgrid, 256, 0, st>>>(se, si);
     ++c->launches;
     if (ev) CK(cudaEventRecord(ev[4], st));
+    const AdvanceArgs adv{c->d_steps, c->d_slab, c->nslot, c->slab_app, c->slab_err};
     if (shape.field) {
         nv.phase("fields");
         const int nsub = shape.nsub;
@@ -649,17 +671,25 @@ pic_status launch_step(pic_ctx *c)
         for (int sub = 0; sub < nsub; ++sub) {
             f.sub = sub;
             f.Ein = c->E[c->ecur]; f.Eout = c->E[c->ecur ^ 1];
+            c->ecur ^= 1;
+            const bool last = sub == nsub - 1;
+            if (c->slot_rows == 1 && nsub == 1) {
+                k_field_1d<<<c->nslot, FIELD1_T, 0, st>>>(f, adv, c->slot_pts);
+                ++c->launches;
+                continue;
+            }
             k_b_half<<<fg, 256, 0, st>>>(f);
             k_e_full<<<fg, 256, 0, st>>>(f);
-            c->ecur ^= 1;
             f.Ein = c->E[c->ecur];
-            k_b_half<<<fg, 256, 0, st>>>(f);
+            if (last && !c->batch) k_b_half_advance<<<fg, 256, 0, st>>>(f, adv);
+            else k_b_half<<<fg, 256, 0, st>>>(f);
             c->launches += 3;
         }
     }
-    const AdvanceArgs adv{c->d_steps, c->d_slab, c->nslot, c->slab_app, c->slab_err};
-    k_advance<<<(c->nslot + 127) / 128, 128, 0, st>>>(adv);
-    ++c->launches;
+    if (!shape.field || (c->batch && shape.nsub > 1)) {
+        k_advance<<<(c->nslot + 127) / 128, 128, 0, st>>>(adv);
+        ++c->launches;
+    }
     CK(cudaGetLastError());
     if (ev) CK(cudaEventRecord(ev[5], st));
     std::swap(c->eA0, c->eB0); std::swap(c->eA1, c->eB1);
@@ -811,6 +841,9 @@ pic_status ctx_create(pic_ctx **out, int nslot, int slot_cells, int slot_pts, in
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) { pic_status r = cuda_fail(c, e, "device query"); delete c; return r; }
+
+    c->teams = c->ncell * TEAM <= 16 * c->nsm;
+    c->whole = c->ncell <= WHOLE_CELLS && c->ncell <= 2 * c->nsm;
 
     size_t need = arena_need(c->ncell, c->npts, c->nblk, cap_e, cap_i, nslot, c->nrows);
     if (arena) {
@@ -1324,10 +1357,10 @@ pic_status tune_step(pic_ctx *c, int n, int &k)
         c->tuned.push_back(pic_ctx::Tuned{c->cap_ce, c->cap_ci, c->wpc, {0, 0, 0, 0}, 0});
         t = &c->tuned.back();
     }
-    const int top = max_wpc(c->cap_ce, c->cap_ci);
+    const int top = max_wpc(c, c->cap_ce, c->cap_ci);
     int shapes = 0, first = 0;
     while (shapes < 4 && (1 << shapes) <= top) ++shapes;
-    if (team_warps(c->cap_ce, c->cap_ci) > 1) {          // a team has one shape
+    if (team_warps(c, c->cap_ce, c->cap_ci) > 1) {          // a team has one shape
         first = 2;
         shapes = 1;
     }
@@ -1415,12 +1448,14 @@ pic_status step_chunk(pic_ctx *c, int n)
 {
     pic_status r = PIC_OK;
     // size the per-warp staging for the cells of the last sort
-    int cn[NCOUNTERS];
-    CK(cudaMemcpyAsync(cn, c->counters, sizeof(int) * NCOUNTERS, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    if (cn[CNT_MAXE] > 0 || cn[CNT_MAXI] > 0) {
-        r = configure_cell_launch(c, cn + CNT_HIST_E, cn + CNT_HIST_I, cn[CNT_MAXE], cn[CNT_MAXI]);
-        if (r != PIC_OK) return r;
+    if (!c->whole) {
+        int cn[NCOUNTERS];
+        CK(cudaMemcpyAsync(cn, c->counters, sizeof(int) * NCOUNTERS, cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+        if (cn[CNT_MAXE] > 0 || cn[CNT_MAXI] > 0) {
+            r = configure_cell_launch(c, cn + CNT_HIST_E, cn + CNT_HIST_I, cn[CNT_MAXE], cn[CNT_MAXI]);
+            if (r != PIC_OK) return r;
+        }
     }
     int k = 0;
     if (c->autotune) {
@@ -2048,10 +2083,10 @@ pic_status pic_order_check(const uint64_t *key, const uint64_t *id, int n, int r
     // one warp up to 128 or 512 entries, a team above (four warps, whose
     // shares hold 2048; eight for the rest of the range)
     const bool team = rmax == 1024 || n > 512;
-    const int warps = !team ? 1 : (n <= 512 * TEAM ? TEAM : 8);
+    const int warps = !team ? 1 : (n <= 512 * 4 ? 4 : 8);
     const size_t smem = (size_t)n * 8;
     void (*kern)(const unsigned long long *, const unsigned long long *, int, unsigned short *) =
-        warps == 8 ? k_order_check<4096, 8> : warps == TEAM ? k_order_check<2048, TEAM>
+        warps == 8 ? k_order_check<4096, 8> : warps == 4 ? k_order_check<2048, 4>
         : rmax == 128 ? k_order_check<128, 1> : k_order_check<512, 1>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return PIC_ERR_CUDA;

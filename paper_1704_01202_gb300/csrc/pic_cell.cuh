@@ -377,11 +377,13 @@ struct CellMem {
     NewE *nw;                   // [cap_new] in global memory: the team's slice of the scratch
     real *dE;                  // [16] continuum lowering per charge state
     real *Pz;                  // [16] impact-ionization probability per charge
-    real4 *lz;                 // [4][NS] Lotz constants of a charge state (one set per warp): P, 1/P, ln P, a q
+    real4 *lz;                 // [MAX_TEAM][NS] Lotz constants of a charge state (one set per warp): P, 1/P, ln P, a q
     dd *ph;                     // [2 MAXB] photon bin scratch
     int *phc;                   // [MAXB] events per bin so far
     dd *bc;                     // [8] sums a warp hands to its team
 };
+
+constexpr int MAX_TEAM = 8;      // most warps of a team
 
 // shared-memory pieces start on 16 B (FP32) or 32 B (FP64: real4 is 32 B)
 constexpr size_t kSmAlign = sizeof(real4) > 16 ? 32 : 16;
@@ -396,7 +398,7 @@ __host__ __device__ inline size_t cell_mem_bytes(int ce, int ci)
     const int cm = ce > ci ? ce : ci;
     return amem((size_t)ce * sizeof(real4)) + amem((size_t)ce * sizeof(real2)) + amem((size_t)ce * 8) +
            amem((size_t)cm * sizeof(real2)) + amem((size_t)ci * sizeof(real4)) + amem((size_t)ci * sizeof(real2)) +
-           3 * amem((size_t)ci * 4) + 2 * amem(16 * sizeof(real)) + amem(4 * NS * sizeof(real4)) +
+           3 * amem((size_t)ci * 4) + 2 * amem(16 * sizeof(real)) + amem(MAX_TEAM * NS * sizeof(real4)) +
            amem(2 * MAXB * sizeof(dd)) + amem(MAXB * 4) + amem(8 * sizeof(dd));
 }
 
@@ -417,7 +419,7 @@ __device__ inline CellMem carve(char *base, int ce, int ci, NewE *nw)
     m.nw = nw;
     m.dE = (real *)p; p += amem(16 * sizeof(real));
     m.Pz = (real *)p; p += amem(16 * sizeof(real));
-    m.lz = (real4 *)p; p += amem(4 * NS * sizeof(real4));
+    m.lz = (real4 *)p; p += amem(MAX_TEAM * NS * sizeof(real4));
     m.ph = (dd *)p; p += amem(2 * MAXB * sizeof(dd));
     m.phc = (int *)p; p += amem(MAXB * 4);
     m.bc = (dd *)p;

@@ -1136,7 +1136,7 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
 // a list for the next launch.
 // RMAX: the most entries per species a launch stages; TW: warps per cell.
 template <int RMAX, int TW>
-__global__ void __launch_bounds__(TW == 1 ? 256 : 32 * TW, TW == 1 ? 2 : 4) k_cell(CellArgs a)
+__global__ void __launch_bounds__(TW == 1 ? 256 : 32 * TW, TW == 1 ? 2 : 16 / TW) k_cell(CellArgs a)
 {
     extern __shared__ __align__(kSmAlign) char smem[];
     __shared__ Tables T;

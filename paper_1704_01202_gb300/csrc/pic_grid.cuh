@@ -167,30 +167,40 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_final(ScanArgs a)
     const int sp = blockIdx.y;
     const int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
     if (threadIdx.x < NHIST) hs[threadIdx.x] = 0;
+    __shared__ int s_max;
+    if (threadIdx.x == 0) s_max = 0;
+    // (the counts' arrays start at any multiple of 4 bytes)
+    int v[SCAN_ITEMS], sum = 0, mx = 0;
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) v[k] = base + k < a.n ? a.cnt[sp][base + k] : 0;
     const int *before = SELF ? a.cnt[sp] : a.bsum[sp];
     const int nbefore = SELF ? (int)blockIdx.x * SCAN_TILE : (int)blockIdx.x;
     int off = 0;
     for (int k = threadIdx.x; k < nbefore; k += SCAN_T) off += before[k];
-    int tot;
-    block_excl_scan(off, sh, off);
-    int v[SCAN_ITEMS], sum = 0, mx = 0;
+    if (nbefore > 0) block_excl_scan(off, sh, off);
+    else __syncthreads();
+#pragma unroll
     for (int k = 0; k < SCAN_ITEMS; ++k) {
-        v[k] = base + k < a.n ? a.cnt[sp][base + k] : 0;
         sum += v[k];
         mx = max(mx, v[k]);
     }
     // histogram: one shared atomic per distinct bin of a warp
-    for (int k = 0; k < SCAN_ITEMS; ++k) {
-        const int b = v[k] > 0 ? min(32 - __clz(v[k]), NHIST - 1) : 0;
-        const unsigned peers = __match_any_sync(0xffffffffu, b);
-        if (b > 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(hs + b, __popc(peers));
+    if (__any_sync(0xffffffffu, mx > 0)) {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k) {
+            const int b = v[k] > 0 ? min(32 - __clz(v[k]), NHIST - 1) : 0;
+            const unsigned peers = __match_any_sync(0xffffffffu, b);
+            if (b > 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(hs + b, __popc(peers));
+        }
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if ((threadIdx.x & 31) == 0) atomicMax(&s_max, mx);
     }
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(a.maxc[sp], mx);
-    __syncthreads();
-    if (threadIdx.x < NHIST && hs[threadIdx.x]) atomicAdd(a.hist[sp] + threadIdx.x, hs[threadIdx.x]);
+    int tot;
     int ex = block_excl_scan(sum, sh, tot) + off;
+    if (threadIdx.x < NHIST && hs[threadIdx.x]) atomicAdd(a.hist[sp] + threadIdx.x, hs[threadIdx.x]);
+    if (threadIdx.x == 0 && s_max > 0) atomicMax(a.maxc[sp], s_max);
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) a.cs[sp][a.n] = ex + tot;
+#pragma unroll
     for (int k = 0; k < SCAN_ITEMS; ++k) {
         if (base + k < a.n) a.cs[sp][base + k] = ex;
         ex += v[k];
@@ -283,100 +293,106 @@ struct FieldArgs {
     int sub;                 // update index within the step (always 0: nsub = 1)
 };
 
+// half a step of B at grid point p of slab S, from the E at Ein
+__device__ __forceinline__ void b_half_point(const FieldArgs &a, const SlabDev &S, const real *Ein, int p)
+{
+    const int W = S.nx + 1, q = p - S.fld_off;
+    // points past the slab's own (a batch slot wider than the slab) stay zero
+    if (!S.active || !(S.flags & 128u) || a.sub >= S.nsub || q >= W * S.ny) return;
+    const int j = q / W, i = q - j * W;
+    const int jp = (j + 1) % S.ny;
+    const real h = RF(0.5) * S.dt / S.nsub * S.cf;
+    const int n = a.npts;
+    const real *ex = Ein, *ey = Ein + n, *ez = Ein + 2 * n;
+    real *bx = a.B, *by = a.B + n, *bz = a.B + 2 * n;
+    const int o = S.fld_off, r = o + j * W, rp = o + jp * W;
+    bx[p] -= h * (ez[rp + i] - ez[r + i]) / S.dy;
+    if (i < S.nx) {
+        by[p] += h * (ez[r + i + 1] - ez[r + i]) / S.dx;
+        bz[p] -= h * ((ey[r + i + 1] - ey[r + i]) / S.dx - (ex[rp + i] - ex[r + i]) / S.dy);
+    }
+}
+
+// a step of E at grid point p of slab S, Ein to Eout
+__device__ __forceinline__ void e_full_point(const FieldArgs &a, const SlabDev &S, int p)
+{
+    const int n = a.npts;
+    const real *exi = a.Ein, *eyi = a.Ein + n, *ezi = a.Ein + 2 * n;
+    real *exo = a.Eout, *eyo = a.Eout + n, *ezo = a.Eout + 2 * n;
+    const int W = S.nx + 1, q = p - S.fld_off;
+    if (!S.active || !(S.flags & 128u) || a.sub >= S.nsub || q >= W * S.ny) {
+        exo[p] = exi[p]; eyo[p] = eyi[p]; ezo[p] = ezi[p];
+        return;
+    }
+    const int j = q / W, i = q - j * W;
+    const int jm = (j - 1 + S.ny) % S.ny;
+    const int o = S.fld_off, r = o + j * W, rm = o + jm * W;
+    // Cf: speed of the curl terms; C: c, the velocity unit of J
+    const real dtf = S.dt / S.nsub, C = (real)kCnmPerFs, Cf = S.cf, kap = S.kappa_f;
+    const real *bx = a.B, *by = a.B + n, *bz = a.B + 2 * n;
+    const unsigned long long *Jx = a.J, *Jy = a.J + n, *Jz = a.J + 2 * n;
+    const real sx = S.dx / S.dt, sy = S.ny > 1 ? S.dy / S.dt : C;
+    // fixed point (JFIX) back to real: high and low 32 bits separately
+    auto jv = [&](const unsigned long long *Jc, int idx, real scale) {
+        long long v = (long long)Jc[idx];
+        real hi = (real)(int)(v >> 32) * RF(4294967296.0);
+        real lo = (real)(unsigned)(v & 0xffffffffll);
+        return (hi + lo) * (real)(1.0 / JFIX) * scale;
+    };
+    // the current the update sees: (1/4, 1/2, 1/4) along x over the
+    // component's own points (nx faces for Jx, nx + 1 nodes for Jy, Jz;
+    // nothing beyond the slab) and along y (periodic) in 2D
+    const int rp1 = o + ((j + 1) % S.ny) * W;
+    auto js = [&](const unsigned long long *Jc, int ii, int imax, real scale) {
+        real acc = RF(0.0);
+        for (int b = 0; b < 3; ++b) {
+            if (S.ny == 1 && b != 1) continue;
+            const int rr = b == 0 ? rm : (b == 1 ? r : rp1);
+            const real wy = S.ny == 1 ? RF(1.0) : (b == 1 ? RF(0.5) : RF(0.25));
+            for (int d = -1; d <= 1; ++d) {
+                const int ix = ii + d;
+                if (ix < 0 || ix > imax) continue;
+                acc += wy * (d == 0 ? RF(0.5) : RF(0.25)) * jv(Jc, rr + ix, scale);
+            }
+        }
+        return acc;
+    };
+    auto ey_new = [&](int ii) {
+        return eyi[r + ii] + dtf * (-Cf * (bz[r + ii] - bz[r + ii - 1]) / S.dx - kap * js(Jy, ii, S.nx, sy));
+    };
+    auto ez_new = [&](int ii) {
+        return ezi[r + ii] + dtf * (Cf * ((by[r + ii] - by[r + ii - 1]) / S.dx - (bx[r + ii] - bx[rm + ii]) / S.dy)
+                                    - kap * js(Jz, ii, S.nx, C));
+    };
+    if (i < S.nx)
+        exo[p] = exi[p] + dtf * (Cf * (bz[r + i] - bz[rm + i]) / S.dy - kap * js(Jx, i, S.nx - 1, sx));
+    else
+        exo[p] = exi[p];
+    if (i >= 1 && i < S.nx) {
+        eyo[p] = ey_new(i);
+        ezo[p] = ez_new(i);
+    } else if (i == 0) {
+        real y1 = S.nx > 1 ? ey_new(1) : eyi[r + 1], z1 = S.nx > 1 ? ez_new(1) : ezi[r + 1];
+        eyo[p] = eyi[r + 1] + S.mur * (y1 - eyi[r]);
+        ezo[p] = ezi[r + 1] + S.mur * (z1 - ezi[r]);
+    } else {
+        const int l = S.nx - 1;
+        real yl = l >= 1 ? ey_new(l) : eyi[r + l], zl = l >= 1 ? ez_new(l) : ezi[r + l];
+        eyo[p] = eyi[r + l] + S.mur * (yl - eyi[r + S.nx]);
+        ezo[p] = ezi[r + l] + S.mur * (zl - ezi[r + S.nx]);
+    }
+}
+
 __global__ void k_b_half(FieldArgs a)
 {
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.npts; p += gridDim.x * blockDim.x) {
-        const int s = a.pt_slab[p];
-        const SlabDev &S = a.slabs[s];
-        const int W = S.nx + 1, q = p - S.fld_off;
-        // points past the slab's own (a batch slot wider than the slab) stay zero
-        if (!S.active || !(S.flags & 128u) || a.sub >= S.nsub || q >= W * S.ny) continue;
-        const int j = q / W, i = q - j * W;
-        const int jp = (j + 1) % S.ny;
-        const real h = RF(0.5) * S.dt / S.nsub * S.cf;
-        const int n = a.npts;
-        const real *ex = a.Ein, *ey = a.Ein + n, *ez = a.Ein + 2 * n;
-        real *bx = a.B, *by = a.B + n, *bz = a.B + 2 * n;
-        const int o = S.fld_off, r = o + j * W, rp = o + jp * W;
-        bx[p] -= h * (ez[rp + i] - ez[r + i]) / S.dy;
-        if (i < S.nx) {
-            by[p] += h * (ez[r + i + 1] - ez[r + i]) / S.dx;
-            bz[p] -= h * ((ey[r + i + 1] - ey[r + i]) / S.dx - (ex[rp + i] - ex[r + i]) / S.dy);
-        }
-    }
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.npts; p += gridDim.x * blockDim.x)
+        b_half_point(a, a.slabs[a.pt_slab[p]], a.Ein, p);
 }
 
 __global__ void k_e_full(FieldArgs a)
 {
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.npts; p += gridDim.x * blockDim.x) {
-        const int s = a.pt_slab[p];
-        const SlabDev &S = a.slabs[s];
-        const int n = a.npts;
-        const real *exi = a.Ein, *eyi = a.Ein + n, *ezi = a.Ein + 2 * n;
-        real *exo = a.Eout, *eyo = a.Eout + n, *ezo = a.Eout + 2 * n;
-        const int W = S.nx + 1, q = p - S.fld_off;
-        if (!S.active || !(S.flags & 128u) || a.sub >= S.nsub || q >= W * S.ny) {
-            exo[p] = exi[p]; eyo[p] = eyi[p]; ezo[p] = ezi[p];
-            continue;
-        }
-        const int j = q / W, i = q - j * W;
-        const int jm = (j - 1 + S.ny) % S.ny;
-        const int o = S.fld_off, r = o + j * W, rm = o + jm * W;
-        // Cf: speed of the curl terms; C: c, the velocity unit of J
-        const real dtf = S.dt / S.nsub, C = (real)kCnmPerFs, Cf = S.cf, kap = S.kappa_f;
-        const real *bx = a.B, *by = a.B + n, *bz = a.B + 2 * n;
-        const unsigned long long *Jx = a.J, *Jy = a.J + n, *Jz = a.J + 2 * n;
-        const real sx = S.dx / S.dt, sy = S.ny > 1 ? S.dy / S.dt : C;
-        // fixed point (JFIX) back to real: high and low 32 bits separately
-        auto jv = [&](const unsigned long long *Jc, int idx, real scale) {
-            long long v = (long long)Jc[idx];
-            real hi = (real)(int)(v >> 32) * RF(4294967296.0);
-            real lo = (real)(unsigned)(v & 0xffffffffll);
-            return (hi + lo) * (real)(1.0 / JFIX) * scale;
-        };
-        // the current the update sees: (1/4, 1/2, 1/4) along x over the
-        // component's own points (nx faces for Jx, nx + 1 nodes for Jy, Jz;
-        // nothing beyond the slab) and along y (periodic) in 2D
-        const int rp1 = o + ((j + 1) % S.ny) * W;
-        auto js = [&](const unsigned long long *Jc, int ii, int imax, real scale) {
-            real acc = RF(0.0);
-            for (int b = 0; b < 3; ++b) {
-                if (S.ny == 1 && b != 1) continue;
-                const int rr = b == 0 ? rm : (b == 1 ? r : rp1);
-                const real wy = S.ny == 1 ? RF(1.0) : (b == 1 ? RF(0.5) : RF(0.25));
-                for (int d = -1; d <= 1; ++d) {
-                    const int ix = ii + d;
-                    if (ix < 0 || ix > imax) continue;
-                    acc += wy * (d == 0 ? RF(0.5) : RF(0.25)) * jv(Jc, rr + ix, scale);
-                }
-            }
-            return acc;
-        };
-        auto ey_new = [&](int ii) {
-            return eyi[r + ii] + dtf * (-Cf * (bz[r + ii] - bz[r + ii - 1]) / S.dx - kap * js(Jy, ii, S.nx, sy));
-        };
-        auto ez_new = [&](int ii) {
-            return ezi[r + ii] + dtf * (Cf * ((by[r + ii] - by[r + ii - 1]) / S.dx - (bx[r + ii] - bx[rm + ii]) / S.dy)
-                                        - kap * js(Jz, ii, S.nx, C));
-        };
-        if (i < S.nx)
-            exo[p] = exi[p] + dtf * (Cf * (bz[r + i] - bz[rm + i]) / S.dy - kap * js(Jx, i, S.nx - 1, sx));
-        else
-            exo[p] = exi[p];
-        if (i >= 1 && i < S.nx) {
-            eyo[p] = ey_new(i);
-            ezo[p] = ez_new(i);
-        } else if (i == 0) {
-            real y1 = S.nx > 1 ? ey_new(1) : eyi[r + 1], z1 = S.nx > 1 ? ez_new(1) : ezi[r + 1];
-            eyo[p] = eyi[r + 1] + S.mur * (y1 - eyi[r]);
-            ezo[p] = ezi[r + 1] + S.mur * (z1 - ezi[r]);
-        } else {
-            const int l = S.nx - 1;
-            real yl = l >= 1 ? ey_new(l) : eyi[r + l], zl = l >= 1 ? ez_new(l) : ezi[r + l];
-            eyo[p] = eyi[r + l] + S.mur * (yl - eyi[r + S.nx]);
-            ezo[p] = ezi[r + l] + S.mur * (zl - ezi[r + S.nx]);
-        }
-    }
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.npts; p += gridDim.x * blockDim.x)
+        e_full_point(a, a.slabs[a.pt_slab[p]], p);
 }
 
 // end of a step: every running slab's step count advances; a slab that
@@ -390,6 +406,35 @@ __device__ __forceinline__ void advance_slab(const AdvanceArgs &a, int s)
     if (!a.slabs[s].active) return;
     if (a.slab_err[s]) a.slabs[s].active = 0;
     else a.steps[s] += 1u;
+}
+
+// The second half step of B in 2D (single-slab contexts) and the end of the
+// step: B does not read the step count.
+__global__ void k_b_half_advance(FieldArgs a, AdvanceArgs v)
+{
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.npts; p += gridDim.x * blockDim.x)
+        b_half_point(a, a.slabs[a.pt_slab[p]], a.Ein, p);
+    if (blockIdx.x == 0 && threadIdx.x == 0) advance_slab(v, 0);
+}
+
+// The field update of 1D slabs, a block each (slot_pts grid points), and the
+// end of their step.  A slab's update is a few hundred points three times
+// over; as four launches it took 21 us of a small slab's step, most of it
+// starting and ending, as one 9 (128 cells; 24 slabs of 250 cells 21 -> 11,
+// 20 of up to 2048, 25 -> 26: a block's three passes there cost what the
+// launches did).
+constexpr int FIELD1_T = 512;
+__global__ void __launch_bounds__(FIELD1_T) k_field_1d(FieldArgs a, AdvanceArgs v, int slot_pts)
+{
+    const int s = blockIdx.x, p0 = s * slot_pts;
+    const SlabDev &S = a.slabs[s];
+    for (int p = p0 + (int)threadIdx.x; p < p0 + slot_pts; p += FIELD1_T) b_half_point(a, S, a.Ein, p);
+    __syncthreads();
+    for (int p = p0 + (int)threadIdx.x; p < p0 + slot_pts; p += FIELD1_T) e_full_point(a, S, p);
+    __syncthreads();
+    for (int p = p0 + (int)threadIdx.x; p < p0 + slot_pts; p += FIELD1_T) b_half_point(a, S, a.Eout, p);
+    __syncthreads();
+    if (threadIdx.x == 0) advance_slab(v, s);
 }
 
 __global__ void k_advance(AdvanceArgs a)

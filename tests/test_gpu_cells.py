@@ -57,11 +57,13 @@ def test_cell_sizes_one_step(tables, ppc_e, ppc_i):
     _assert_parity(cfg, st, g, o)
 
 
-@pytest.mark.parametrize("ppc_e,ppc_i,T_e", [(31, 1, 10.0), (33, 32, 2e4), (100, 25, 3e5), (600, 130, 50.0)])
-def test_push_team_and_warp_agree(tables, ppc_e, ppc_i, T_e):
+@pytest.mark.parametrize("ppc_e,ppc_i,T_e", [(31, 1, 10.0), (33, 32, 2e4), (100, 25, 3e5), (128, 128, 30.0),
+                                             (129, 31, 30.0), (300, 500, 30.0), (505, 102, 30.0), (600, 130, 50.0)])
+def test_team_and_warp_agree(tables, ppc_e, ppc_i, T_e):
     """A slab alone has fewer cells than fill the GPU (a block per cell in the
-    push); in a context of 4096 cells the same slab is pushed one warp per
-    cell.  Same state bit for bit, with created electrons, particles leaving
+    cell kernel, staged at the largest size, and in the push); in a context of
+    4096 cells the same slab goes one warp per cell through the tiers of its
+    sizes.  Same state bit for bit, with created electrons, particles leaving
     through the boundaries and moves of more than a cell (T_e = 3e5)."""
     cfg = P.cfg_small_1d(nx=24, ppc_e=ppc_e, ppc_i=ppc_i, T_e_eV=T_e, flags=P.F_ALL, rad_every=1)
     pl = P.Pulse(I_peak_Wcm2=3e17, fwhm_fs=30.0, t_peak_fs=0.0, hv_eV=1700.0, n_bins=2, bandwidth_eV=60.0)
