@@ -252,8 +252,19 @@ CellKernel cell_kernel(const pic_ctx *c, int ce, int ci)
     return std::max(ce, ci) <= 128 ? k_cell<128, 1> : k_cell<512, 1>;
 }
 
+// of tier 0: with many rounds over the cells, the instance that looks ahead
+CellKernel tier0_kernel(const pic_ctx *c)
+{
+    const CellKernel k = cell_kernel(c, c->cap_ce, c->cap_ci);
+    return k == k_cell<128, 1> && c->ncell >= 8LL * c->grid_main * c->wpc ? k_cell<128, 1, true> : k;
+}
+
 // shared memory of a CTA of wpc warps (wpc / team_warps cells)
-size_t cell_smem(const pic_ctx *c, int ce, int ci, int wpc) { return cell_mem_bytes(ce, ci) * (wpc / team_warps(c, ce, ci)); }
+size_t cell_smem(const pic_ctx *c, int ce, int ci, int wpc)
+{
+    const int tw = team_warps(c, ce, ci);
+    return cell_mem_bytes(ce, ci, tw) * (wpc / tw);
+}
 
 // largest warps per CTA of the cell kernel whose staging fits 200 KB, at
 // most 8 and at most what the instance's launch bounds allow; a team is a
@@ -261,7 +272,7 @@ size_t cell_smem(const pic_ctx *c, int ce, int ci, int wpc) { return cell_mem_by
 int max_wpc(const pic_ctx *c, int ce, int ci)
 {
     if (team_warps(c, ce, ci) > 1) return team_warps(c, ce, ci);
-    const size_t per = cell_mem_bytes(ce, ci);
+    const size_t per = cell_mem_bytes(ce, ci, 1);
     int lim = 8;
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, cell_kernel(c, ce, ci)) == cudaSuccess && fa.maxThreadsPerBlock >= 32)
@@ -285,7 +296,7 @@ pic_status cell_smem_attr(pic_ctx *c)
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const size_t m = std::max(std::max(c->smem_main, c->smem_t1), std::max(c->smem_t2, c->smem_big));
-    for (CellKernel k : {k_cell<128, 1>, k_cell<512, 1>, k_cell<2048, TEAM>}) {
+    for (CellKernel k : {k_cell<128, 1>, k_cell<128, 1, true>, k_cell<512, 1>, k_cell<2048, TEAM>}) {
         cudaFuncAttributes fa{};
         CK(cudaFuncGetAttributes(&fa, k));
         const size_t lim = optin > (int)fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : m;
@@ -302,6 +313,10 @@ int best_wpc(pic_ctx *c, int ce, int ci)
 {
     if (cell_smem_attr(c) != PIC_OK) return max_wpc(c, ce, ci);
     if (team_warps(c, ce, ci) > 1) return team_warps(c, ce, ci);
+    // few rounds over the cells: small CTAs share them out more evenly (6000
+    // cells 119 us a step at 8 warps, 113 at 2; 4096 76 and 72); from 13
+    // rounds on 8 warps, in step on the same code, are faster (396 and 440)
+    if (c->ncell < 4 * 16 * c->nsm && max_wpc(c, ce, ci) >= 2) return 2;
     int best = 1, best_warps = 0;
     for (int w = 1; w <= max_wpc(c, ce, ci); ++w) {
         int occ = 0;
@@ -609,7 +624,7 @@ pic_status launch_step(pic_ctx *c)
     if (c->cell_ev_on) CK(cudaEventRecord(c->cell_ev[0], st));
     nv.phase("collisions and atomic processes");
     CellArgs a0 = cell_args(c, TIER0);
-    cell_kernel(c, c->cap_ce, c->cap_ci)<<<c->grid_main, c->wpc * 32, c->smem_main, st>>>(a0);
+    tier0_kernel(c)<<<c->grid_main, c->wpc * 32, c->smem_main, st>>>(a0);
     if (c->t1_ce) {
         CellArgs a1 = cell_args(c, TIER1);
         cell_kernel(c, c->t1_ce, c->t1_ci)<<<c->grid_t1, c->t1_wpc * 32, c->smem_t1, st>>>(a1);
@@ -933,7 +948,7 @@ pic_status ctx_create(pic_ctx **out, int nslot, int slot_cells, int slot_pts, in
     } while (0);
     pic_status rc = PIC_OK;
     if (e != cudaSuccess) { rc = cuda_fail(c, e, "init copies"); pic_free(c); return rc; }
-    c->smem_big = cell_mem_bytes(BIG_CE, BIG_CI);
+    c->smem_big = cell_mem_bytes(BIG_CE, BIG_CI, TEAM);
     c->grid_big = cell_grid(c, 1, TEAM, BIG_CE, BIG_CI);
     e = cudaFuncSetAttribute(k_begin, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * 8);
     if (e != cudaSuccess) { rc = cuda_fail(c, e, "begin attribute"); pic_free(c); return rc; }

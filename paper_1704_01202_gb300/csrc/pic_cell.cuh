@@ -369,6 +369,7 @@ struct CellMem {
     unsigned long long *eid;    // [cap_ce]
     real2 *ew;                 // [max(cap_ce, cap_ci)] scratch: sort words; kinetic energy and w beta of each
                                 //   electron; weight taken by recombination
+    real4 *rn;                 // [cap_ce] e-i collisions' draws (launches of small cells, coll_draws_staged)
     real4 *iu;                 // [cap_ci] ux uy uz zfrac
     real2 *ipos;               // [cap_ci]
     int *ist;                   // [cap_ci] Z | nK << 8
@@ -377,32 +378,38 @@ struct CellMem {
     NewE *nw;                   // [cap_new] in global memory: the team's slice of the scratch
     real *dE;                  // [16] continuum lowering per charge state
     real *Pz;                  // [16] impact-ionization probability per charge
-    real4 *lz;                 // [MAX_TEAM][NS] Lotz constants of a charge state (one set per warp): P, 1/P, ln P, a q
+    real4 *lz;                 // [TW][LOTZ_SETS][NS] Lotz constants of a charge state (a warp's four sets): P, 1/P, ln P, a q
     dd *ph;                     // [2 MAXB] photon bin scratch
     int *phc;                   // [MAXB] events per bin so far
     dd *bc;                     // [8] sums a warp hands to its team
 };
 
-constexpr int MAX_TEAM = 8;      // most warps of a team
+constexpr int LOTZ_SETS = 4;     // a warp
 
 // shared-memory pieces start on 16 B (FP32) or 32 B (FP64: real4 is 32 B)
 constexpr size_t kSmAlign = sizeof(real4) > 16 ? 32 : 16;
 __host__ __device__ inline size_t amem(size_t x) { return (x + kSmAlign - 1) & ~(kSmAlign - 1); }
 
-// Shared memory of a team staging up to ce electrons and ci ions.  The
+// The launches that stage at most 128 entries, a warp a cell, form the draws of the e-i
+// collisions before the chains of collisions (see there): 16 bytes more an
+// electron, which would cost the larger ones resident warps.
+__host__ __device__ constexpr bool coll_draws_staged(int ce, int ci, int tw) { return ce <= 128 && ci <= 128 && tw == 1; }
+
+// Shared memory of a team of tw warps staging up to ce electrons and ci ions.  The
 // electrons a cell creates in a step (up to 3 per ion: impact, photo- and
 // Auger ionization) are rare; they live in the team's slice of a global
 // scratch, which keeps the staging of large cells small.
-__host__ __device__ inline size_t cell_mem_bytes(int ce, int ci)
+__host__ __device__ inline size_t cell_mem_bytes(int ce, int ci, int tw)
 {
     const int cm = ce > ci ? ce : ci;
     return amem((size_t)ce * sizeof(real4)) + amem((size_t)ce * sizeof(real2)) + amem((size_t)ce * 8) +
-           amem((size_t)cm * sizeof(real2)) + amem((size_t)ci * sizeof(real4)) + amem((size_t)ci * sizeof(real2)) +
-           3 * amem((size_t)ci * 4) + 2 * amem(16 * sizeof(real)) + amem(MAX_TEAM * NS * sizeof(real4)) +
+           amem((size_t)cm * sizeof(real2)) + (coll_draws_staged(ce, ci, tw) ? amem((size_t)ce * sizeof(real4)) : 0) +
+           amem((size_t)ci * sizeof(real4)) + amem((size_t)ci * sizeof(real2)) +
+           3 * amem((size_t)ci * 4) + 2 * amem(16 * sizeof(real)) + amem(tw * LOTZ_SETS * NS * sizeof(real4)) +
            amem(2 * MAXB * sizeof(dd)) + amem(MAXB * 4) + amem(8 * sizeof(dd));
 }
 
-__device__ inline CellMem carve(char *base, int ce, int ci, NewE *nw)
+__device__ inline CellMem carve(char *base, int ce, int ci, int tw, NewE *nw)
 {
     CellMem m;
     const int cm = ce > ci ? ce : ci;
@@ -411,6 +418,8 @@ __device__ inline CellMem carve(char *base, int ce, int ci, NewE *nw)
     m.epos = (real2 *)p; p += amem((size_t)ce * sizeof(real2));
     m.eid = (unsigned long long *)p; p += amem((size_t)ce * 8);
     m.ew = (real2 *)p; p += amem((size_t)cm * sizeof(real2));
+    m.rn = (real4 *)p;
+    if (coll_draws_staged(ce, ci, tw)) p += amem((size_t)ce * sizeof(real4));
     m.iu = (real4 *)p; p += amem((size_t)ci * sizeof(real4));
     m.ipos = (real2 *)p; p += amem((size_t)ci * sizeof(real2));
     m.ist = (int *)p; p += amem((size_t)ci * 4);
@@ -419,7 +428,7 @@ __device__ inline CellMem carve(char *base, int ce, int ci, NewE *nw)
     m.nw = nw;
     m.dE = (real *)p; p += amem(16 * sizeof(real));
     m.Pz = (real *)p; p += amem(16 * sizeof(real));
-    m.lz = (real4 *)p; p += amem(MAX_TEAM * NS * sizeof(real4));
+    m.lz = (real4 *)p; p += amem(tw * LOTZ_SETS * NS * sizeof(real4));
     m.ph = (dd *)p; p += amem(2 * MAXB * sizeof(dd));
     m.phc = (int *)p; p += amem(MAXB * 4);
     m.bc = (dd *)p;

@@ -164,15 +164,14 @@ __device__ __noinline__ void stage_therm(const CellMem &m, const CellCtx &c, int
 }
 
 // ---- EOS-clamped three-body recombination (Sec. IV) ----
-// Run by one warp; a team's other warps join for the last pass, the
-// correction of every electron's energy (see recombine_apply).  Returns
-// whether events happened, with that pass's factor in delta.
-__device__ __noinline__ bool stage_recombine(const CellArgs &a, const CellMem &m, const Tables &T, const SlabDev &S,
-                                             const CellCtx &c, int lane, real Wnew_imp, WarpTally &wt, real &delta)
+// How many events the clamp asks for, before what the cell can give; Wex:
+// the electrons' weight.  By one warp.
+__device__ __forceinline__ int recombine_wanted(const CellArgs &a, const CellMem &m, real E_bulk, const CellCtx &c, int lane,
+                                                real Wnew_imp, real &Wex)
 {
     const int ne = c.ne, ni = c.ni;
-    const real wi = c.wi, MC2 = (real)kMeC2;
-    real zb, Wb2, Kb2, Wex;
+    const real MC2 = (real)kMeC2;
+    real zb, Wb2, Kb2;
     if (c.have_sums) {
         // every electron is bulk: the sums of the moments and ionization
         // stages, which the ionization payment changed by a known amount
@@ -190,16 +189,25 @@ __device__ __noinline__ bool stage_recombine(const CellArgs &a, const CellMem &m
             real4 u = m.eu[k];
             real ke = MC2 * gm1(u.x, u.y, u.z);
             pwx += u.w;
-            if (S.E_bulk <= RF(0.0) || ke < S.E_bulk) { pwb += u.w; pkb = dd_addf(pkb, u.w * ke); }
+            if (E_bulk <= RF(0.0) || ke < E_bulk) { pwb += u.w; pkb = dd_addf(pkb, u.w * ke); }
         }
         Wb2 = wsum_f(pwb) + Wnew_imp;
         Kb2 = dd_f(wsum_dd(pkb));
         Wex = wsum_f(pwx);
     }
     const real Te2 = Wb2 > RF(0.0) ? (RF(2.0) / RF(3.0)) * Kb2 / Wb2 : RF(0.0);
-    const real zeos = eos_lookup(*a.eos, c.n_i, Te2);
-    int Kev = zb > zeos ? (int)r_floor((zb - zeos) * ni + RF(0.5)) : 0;
-    if (Kev <= 0) return false;
+    const real zeos = eos_lookup(*a.eos, c.n_i, Te2, lane);
+    return zb > zeos ? (int)r_floor((zb - zeos) * ni + RF(0.5)) : 0;
+}
+
+// The events themselves (in a fifth of the cells of a solid-density plasma,
+// so out of line), by one warp; a team's other warps join for the last pass,
+// the correction of every electron's energy (recombine_apply).  Returns
+// whether events happened, with that pass's factor in delta.
+__device__ __noinline__ bool stage_recombine(const CellArgs &a, const CellMem &m, const Tables &T, real E_bulk, real wi,
+                                             int ne, int ni, int lane, int Kev, real Wex, WarpTally &wt, real &delta)
+{
+    const real MC2 = (real)kMeC2;
     int pel = 0;
     for (int k = lane; k < ni; k += 32) pel += m.ist[k] & 0xff;
     const int elig = wsum_i(pel);
@@ -262,7 +270,7 @@ __device__ __noinline__ bool stage_recombine(const CellArgs &a, const CellMem &m
     for (int k = lane; k < ne; k += 32) {
         real4 u = m.eu[k];
         real ke = MC2 * gm1(u.x, u.y, u.z);
-        if (S.E_bulk <= RF(0.0) || ke < S.E_bulk) pkr = dd_addf(pkr, (u.w - take[k]) * ke);
+        if (E_bulk <= RF(0.0) || ke < E_bulk) pkr = dd_addf(pkr, (u.w - take[k]) * ke);
     }
     const real Krem = dd_f(wsum_dd(pkr));
     if (!(Krem > RF(0.0))) return false;
@@ -528,9 +536,9 @@ __device__ __forceinline__ void team_sync()
     else __syncthreads();
 }
 
-template <int RMAX, int TW>
+template <int RMAX, int TW, bool EARLY>
 __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &T, int g, int warp, int lane,
-                             WarpTally &wt, LaneTally &lt)
+                             WarpTally &wt, LaneTally &lt, const int *next)
 {
     constexpr int nt = 32 * TW;
     const int t0 = TW == 1 ? lane : warp * 32 + lane;
@@ -583,12 +591,24 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
         const RecKeys K{a.e1 + e0, true, seed, step};
         for (int k = t0; k < ne; k += nt) prefetch_l2(a.e0 + e0 + k);
         const unsigned mask = order_cell<RMAX, TW>(K, words, words + ne, ne, warp, lane);
-        for (int k = t0; k < ne; k += nt) {
-            const int sl = (int)(words[k] & mask);
-            const real4 P0 = a.e0[e0 + sl], P1 = a.e1[e0 + sl];
-            m.eu[k] = make_real4(P0.z, P0.w, P1.x, P1.y);
-            m.epos[k] = make_real2(P0.x, P0.y);
-            m.eid[k] = rec_eid(P1);
+        for (int b0 = 0; b0 < ne; b0 += 2 * nt) {         // two records a thread in flight
+            real4 P0[2], P1[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int k = b0 + j * nt + t0;
+                if (k >= ne) break;
+                const int sl = (int)(words[k] & mask);
+                P0[j] = a.e0[e0 + sl];
+                P1[j] = a.e1[e0 + sl];
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int k = b0 + j * nt + t0;
+                if (k >= ne) break;
+                m.eu[k] = make_real4(P0[j].z, P0[j].w, P1[j].x, P1[j].y);
+                m.epos[k] = make_real2(P0[j].x, P0[j].y);
+                m.eid[k] = rec_eid(P1[j]);
+            }
         }
         team_sync<TW>();
     }
@@ -606,7 +626,6 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
         team_sync<TW>();
     }
     }
-    if constexpr (TW == 1) __syncthreads();
 
     if (on && rad && S.rt) {
     // ---- transport mode: the energy the radiation field gave up to (or
@@ -712,7 +731,7 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
         auto ee = [&](int pa, int pb, real dtc) {
             const real4 A = m.eu[pa], B = m.eu[pb];
             const U4 r = draw(seed, m.eid[pa], step, PU_COLL_EE);
-            const Collided q = binary_collision(A, B, RF(1.0), RF(1.0), -RF(1.0), -RF(1.0), A.w, B.w, n_e, lnL, dtc, r);
+            const Collided q = binary_collision(A, B, RF(1.0), RF(1.0), -RF(1.0), -RF(1.0), A.w, B.w, n_e, lnL, dtc, coll_draw(r));
             lt.ee += q.hit;
             m.eu[pa] = q.a;
             m.eu[pb] = q.b;
@@ -728,7 +747,14 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
     }
     team_sync<TW>();
     }
+    // the cell this warp takes next: where its records are, for a prefetch
+    // into L2 after this cell's e-i collisions
+    [[maybe_unused]] int pe0 = 0, pe1 = 0, pi0 = 0, pi1 = 0;
     if constexpr (TW == 1) __syncthreads();     // the e-i code next: warps in step, as elsewhere
+    if constexpr (EARLY) {
+        const int gn = *next + warp;
+        if (gn < a.ncell) { pe0 = a.cs_e[gn]; pe1 = a.cs_e[gn + 1]; pi0 = a.cs_i[gn]; pi1 = a.cs_i[gn + 1]; }
+    }
 
     if (on) {
     if ((flags & 2u) && ne >= 1 && ni >= 1) {
@@ -736,6 +762,19 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
         // shorter meets t, t + nshort, ... of the longer, one after another,
         // and no other thread touches any of them
         if (ne >= ni) {
+            // The chains keep as many lanes busy as there are ions (16 to 20
+            // of 32 in the 2D workloads); the draws, half of a collision's
+            // instructions, depend on the electron alone, so one warp forms
+            // them first with all its lanes.
+            constexpr bool STAGED = RMAX <= 128 && TW == 1;
+            if constexpr (STAGED) {
+                for (int pe = lane; pe < ne; pe += 32) {
+                    const CollDraw d = coll_draw(draw(seed, m.eid[pe], step, PU_COLL_EI));
+                    m.rn[pe] = make_real4(d.a, d.c, d.sphi, d.cphi);
+                    m.ew[pe].x = d.r3;
+                }
+                __syncwarp();
+            }
             for (int pi = t0; pi < ni; pi += nt) {
                 real4 B = m.iu[pi];
                 const real q = (real)(m.ist[pi] & 0xff) + B.w;
@@ -743,8 +782,14 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
                 for (int pe = pi; pe < ne; pe += ni) {
                     const real4 A = m.eu[pe];
                     const real npair = n_i * r_fmax(A.w, wi) / wi;
-                    const U4 r = draw(seed, m.eid[pe], step, PU_COLL_EI);
-                    const Collided c = binary_collision(A, B, RF(1.0), mi, -RF(1.0), q, A.w, wi, npair, lnL, dt, r);
+                    CollDraw d;
+                    if constexpr (STAGED) {
+                        const real4 v = m.rn[pe];
+                        d = CollDraw{v.x, v.y, v.z, v.w, m.ew[pe].x};
+                    } else {
+                        d = coll_draw(draw(seed, m.eid[pe], step, PU_COLL_EI));
+                    }
+                    const Collided c = binary_collision(A, B, RF(1.0), mi, -RF(1.0), q, A.w, wi, npair, lnL, dt, d);
                     lt.ei += c.hit;
                     m.eu[pe] = c.a;
                     B = c.b;
@@ -760,7 +805,7 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
                     const real q = (real)(m.ist[pi] & 0xff) + B.w;
                     const real npair = n_e * r_fmax(A.w, wi) / A.w;
                     const U4 r = draw(seed, (unsigned long long)m.iid[pi], step, PU_COLL_IE);
-                    const Collided c = binary_collision(A, B, RF(1.0), mi, -RF(1.0), q, A.w, wi, npair, lnL, dt, r);
+                    const Collided c = binary_collision(A, B, RF(1.0), mi, -RF(1.0), q, A.w, wi, npair, lnL, dt, coll_draw(r));
                     lt.ei += c.hit;
                     A = c.a;
                     m.iu[pi] = c.b;
@@ -833,6 +878,12 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
 
     }
     if constexpr (TW == 1) __syncthreads();
+    if constexpr (EARLY) {
+        constexpr int PER = 128 / sizeof(real4);
+        const bool elec = lane < 24;
+        const int k = (elec ? pe0 : pi0) + PER * (elec ? lane % 12 : lane % 4);
+        if (k < (elec ? pe1 : pi1)) prefetch_l2((elec ? (lane < 12 ? a.e0 : a.e1) : (lane < 28 ? a.i0 : a.i1)) + k);
+    }
 
     if (on) {
     // ---- Lotz impact ionization, cell-average probability (Eq. 3) ----
@@ -901,53 +952,60 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
             Kt = m.bc[2];
             nhot = (int)m.bc[3].hi;
         }
+        // Charge states side by side: with a few hot electrons the lanes form
+        // groups of 8, 16 or 32, a charge state each (what the lanes beyond
+        // nhot would add to a sum's tree is zero).
         const real cfac = (real)(kCcmPerFs) * dt * nref;
-        real4 *lz = m.lz + (TW == 1 ? 0 : warp * NS);
-        int zi = 0;
-        for (int z = 0; z < ZNUC; ++z) {
-            if (!(pmask & (1u << z))) continue;
-            if (TW > 1 && (zi++ % TW) != warp) continue;
+        real4 *lz = m.lz + (TW == 1 ? 0 : warp * LOTZ_SETS * NS);
+        const int G = nhot <= 8 ? 8 : (nhot <= 16 ? 16 : 32), gl = lane & (G - 1), gi = lane / G, per = 32 / G;
+        unsigned zs = pmask;                         // charge states to come
+        auto drop = [](unsigned v, int n) { for (int j = 0; j < n; ++j) v &= v - 1u; return v; };
+        if (TW > 1) zs = drop(zs, warp * per);
+        for (; zs; zs = drop(zs, TW * per)) {
+            // the group's charge state: the gi-th of them (-1: none)
+            const int z = __ffs(drop(zs, gi)) - 1;
             // Lotz constants of charge state z (lowest-energy configuration):
             // lowered binding P, 1/P, ln P, a * occupation (0: empty subshell)
-            if (lane < NS) {
-                const int o = subshell_occ(ZNUC - z, lane);
+            if (gl < NS) {
+                const int o = z >= 0 ? subshell_occ(ZNUC - z, gl) : 0;
                 real4 v = make_real4(RF(0.0), RF(0.0), RF(0.0), RF(0.0));
                 if (o > 0) {
-                    const real P = lowered_binding(T, z, lane, m.dE[z]);
-                    v = make_real4(P, RF(1.0) / P, r_log(P), T.lotz_a[lane] * (real)o);
+                    const real P = lowered_binding(T, z, gl, m.dE[z]);
+                    v = make_real4(P, RF(1.0) / P, r_log(P), T.lotz_a[gl] * (real)o);
                 }
-                lz[lane] = v;
+                lz[gi * NS + gl] = v;
             }
             __syncwarp();
-            // the lowest lowered binding of the charge state: electrons at
-            // or below it ionize no subshell and add nothing to the sum
-            real Pmin = RF(3.0e38);
-#pragma unroll
-            for (int sh = 0; sh < NS; ++sh)
-                if (lz[sh].w > RF(0.0)) Pmin = r_fmin(Pmin, lz[sh].x);
             // fast log / exp: a few ulp on a probability; only a decision
             // within that of its threshold could flip
             dd pr = dd_zero();
-            for (int k = lane; k < nhot; k += 32) {
+            for (int k = gl; k < nhot; k += G) {
                 const real2 q = ew[k];
-                if (!(q.x > Pmin)) continue;
                 const real E = q.x, lnE = r_flog(E), invE = RF(1.0) / E;
                 real sig = RF(0.0);
+                bool any = false;
 #pragma unroll
                 for (int sh = 0; sh < NS; ++sh) {
-                    const real4 L = lz[sh];
+                    const real4 L = lz[gi * NS + sh];
                     if (L.w > RF(0.0) && E > L.x) {
                         const real x = E * L.y;
                         sig += L.w * (lnE - L.z) * (invE * L.y) *
                                (RF(1.0) - T.lotz_b[sh] * r_fexp(-T.lotz_c[sh] * (x - RF(1.0))));
+                        any = true;
                     }
                 }
-                pr = dd_addf(pr, q.y * sig);
+                // at or below the lowest binding of the charge state: nothing
+                if (any) pr = dd_addp(pr, q.y, sig);
             }
-            // no hot electron: the sum is zero
-            real P = nhot > 0 ? cfac * dd_f(wsum_dd(pr)) : RF(0.0);
-            if (lane == 0) m.Pz[z] = P;
-            if (P > RF(1.0) && lane == 0) wt.cnt[C_PGT1]++;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (o < G) {
+                    dd t{__shfl_xor_sync(FULL, pr.hi, o), __shfl_xor_sync(FULL, pr.lo, o)};
+                    pr = dd_add(pr, t);
+                }
+            const real P = cfac * dd_f(pr);
+            if (gl == 0 && z >= 0) m.Pz[z] = P;
+            wt.cnt[C_PGT1] += __popc(__ballot_sync(FULL, gl == 0 && z >= 0 && P > RF(1.0)));
             __syncwarp();
         }
         team_sync<TW>();
@@ -1022,9 +1080,8 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
 
     if (on) {
     if ((flags & 8u) && ni >= 1) {
-        CellCtx cc;
-        cc.lc = lc; cc.ne = ne; cc.ni = ni;
-        cc.step = step; cc.seed = seed; cc.wi = wi; cc.n_i = n_i; cc.nref = nref;
+        CellCtx cc;                       // (inline: in registers)
+        cc.ne = ne; cc.ni = ni; cc.n_i = n_i;
         cc.have_sums = all_bulk && ionized;
         cc.K_after = dd_sub(Kt, paid_cell);
         cc.W_e = We_cell;
@@ -1032,7 +1089,9 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
         real delta = RF(0.0);
         bool rec = false;
         if (w0) {
-            rec = stage_recombine(a, m, T, S, cc, lane, Wnew_imp, wt, delta);
+            real Wex;
+            const int Kev = recombine_wanted(a, m, E_bulk, cc, lane, Wnew_imp, Wex);
+            if (Kev > 0) rec = stage_recombine(a, m, T, E_bulk, wi, ne, ni, lane, Kev, Wex, wt, delta);
             if (TW > 1 && lane == 0) m.bc[5] = dd{delta, rec ? RF(1.0) : RF(0.0)};
         }
         if constexpr (TW > 1) {
@@ -1130,36 +1189,50 @@ __device__ void process_cell(const CellArgs &a, const CellMem &m, const Tables &
 // keeps its state in registers through its chain of collisions.  Against the
 // 64-bit sort, slot-ordered staging, one reduction per sum and collisions
 // called by reference: 2048 x 256 cells of 64 e + 16 i, 42 M particles, 6.94
-// -> 5.40 ms a step; 512 x 64 cells 511 -> 397 us.
+// -> 5.40 ms a step; 512 x 64 cells 511 -> 397 us.  With the Lotz sums of
+// several charge states side by side, the recombination clamp inline, the
+// e-i draws formed ahead of their chains and the next cell's records
+// prefetched: 4.88 ms and 364 us.  Two CTAs of 8 warps an SM: 6 to 10 warps a
+// CTA at 80 to 112 registers (18 to 24 warps an SM) take 5.2 to 6.0 ms, one
+// CTA of 16 warps 5.4.
 // Each round the block takes one cell per team from a shared counter.
 // Cells whose population exceeds this launch's shared-memory capacity go to
 // a list for the next launch.
 // RMAX: the most entries per species a launch stages; TW: warps per cell.
-template <int RMAX, int TW>
+// EARLY: a block takes its next round's cells while it computes this one's
+// and prefetches their records into L2; for launches of many rounds over all
+// cells (with few rounds, a block that took its cells early leaves them
+// waiting while others are idle).
+template <int RMAX, int TW, bool EARLY = false>
 __global__ void __launch_bounds__(TW == 1 ? 256 : 32 * TW, TW == 1 ? 2 : 16 / TW) k_cell(CellArgs a)
 {
     extern __shared__ __align__(kSmAlign) char smem[];
     __shared__ Tables T;
-    __shared__ int round_base;
+    __shared__ int s_next;               // first cell of the block's next round
     const int total = a.list ? *a.n_list : a.ncell;
     if (total == 0) return;              // a tier no cell needs
     for (int k = threadIdx.x; k < (int)(sizeof(Tables) / sizeof(real)); k += blockDim.x)
         ((real *)&T)[k] = ((const real *)a.tab)[k];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nteam = TW == 1 ? blockDim.x >> 5 : 1;
     const int team = TW == 1 ? warp : 0;
-    CellMem m = carve(smem + (size_t)team * cell_mem_bytes(a.cap_ce, a.cap_ci), a.cap_ce, a.cap_ci,
+    CellMem m = carve(smem + (size_t)team * cell_mem_bytes(a.cap_ce, a.cap_ci, TW), a.cap_ce, a.cap_ci, TW,
                       a.nw + ((size_t)blockIdx.x * nteam + team) * a.cap_new);
     WarpTally wt;
     LaneTally lt{0, 0, 0, 0};
     wt.slab = -1;
     wt.ion = wt.ka = wt.esc = wt.rt = dd_zero();
     for (int q = 0; q < NCOUNT; ++q) wt.cnt[q] = 0;
+    if (EARLY && threadIdx.x == 0) s_next = atomicAdd(a.work, nteam);
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) round_base = atomicAdd(a.work, nteam);
-        __syncthreads();
-        const int base = round_base;
+        if (!EARLY && threadIdx.x == 0) s_next = atomicAdd(a.work, nteam);
+        if (!EARLY) __syncthreads();
+        const int base = s_next;
         if (base >= total) break;
+        if (EARLY) {
+            __syncthreads();
+            if (threadIdx.x == 0) s_next = atomicAdd(a.work, nteam);
+        }
         int g = -1;
         if (base + team < total) {
             g = a.list ? a.list[base + team] : base + team;
@@ -1180,7 +1253,7 @@ __global__ void __launch_bounds__(TW == 1 ? 256 : 32 * TW, TW == 1 ? 2 : 16 / TW
                 g = -1;
             }
         }
-        process_cell<RMAX, TW>(a, m, T, g, warp, lane, wt, lt);
+        process_cell<RMAX, TW, EARLY>(a, m, T, g, warp, lane, wt, lt, &s_next);
     }
     tally_flush(a, wt, lt, lane);
 }

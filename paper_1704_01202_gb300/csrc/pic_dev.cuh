@@ -393,14 +393,23 @@ __device__ __forceinline__ int subshell_occ(int nb, int s)
     return t <= 0 ? 0 : (t < cap_of(s) ? t : cap_of(s));
 }
 
-// EOS table, bilinear, clamped
-__device__ __forceinline__ real eos_lookup(const EosTable &T, real n, real t)
+// EOS table, bilinear, clamped; by a warp, the same arguments in every
+// lane: the grid interval is found 32 entries at a time (two dependent loads
+// for up to 1024 entries, against ten of a bisection)
+__device__ __forceinline__ real eos_lookup(const EosTable &T, real n, real t, int lane)
 {
-    auto locate = [](const real *g, int m, real x, int &i0) -> real {
+    auto locate = [lane](const real *g, int m, real x, int &i0) -> real {
         if (m == 1 || x <= g[0]) { i0 = 0; return RF(0.0); }
         if (x >= g[m - 1]) { i0 = m - 2; return RF(1.0); }
-        int lo = 0, hi = m - 1;
-        while (hi - lo > 1) { int md = (lo + hi) >> 1; if (g[md] <= x) lo = md; else hi = md; }
+        const int step = (m + 31) >> 5;                 // entries lane * step: the last at or below x
+        const int c = lane * step;
+        int lo = (__popc(__ballot_sync(0xffffffffu, c < m && g[c < m ? c : 0] <= x)) - 1) * step;
+        lo = lo > 0 ? lo : 0;
+        if (step > 1) {
+            const int f = lo + lane;
+            lo += __popc(__ballot_sync(0xffffffffu, lane < step && f < m && g[f < m ? f : 0] <= x)) - 1;
+        }
+        lo = min(max(lo, 0), m - 2);
         i0 = lo;
         return (x - g[lo]) / (g[lo + 1] - g[lo]);
     };
@@ -461,11 +470,28 @@ __device__ __forceinline__ real dot3(real ax, real ay, real az, real bx, real by
     return r_fma(az, bz, r_fma(ax, bx, r_mul(ay, by)));
 }
 
+// What a collision draws: the normal variate of the deflection as two
+// factors (Box-Muller), the azimuth, the acceptance uniform.
+struct CollDraw { real a, c, sphi, cphi, r3; };
+
+__device__ __forceinline__ CollDraw coll_draw(U4 rnd)
+{
+    CollDraw d;
+    d.a = r_sqrt(r_mul(-RF(2.0), r_log(u01(rnd.x))));
+    d.c = r_cospi(r_mul(RF(2.0), u01(rnd.y)));
+    r_sincospi(r_mul(RF(2.0), u01(rnd.z)), &d.sphi, &d.cphi);
+    d.r3 = u01(rnd.w);
+    return d;
+}
+
+__device__ __forceinline__ CollDraw coll_draw(CollDraw d) { return d; }
+
+// Draw: the random words, or what coll_draw made of them before
+template <class Draw>
 __device__ __forceinline__ Collided binary_collision(real4 ua, real4 ub, real ma, real mb, real qa, real qb,
-                                                     real wa, real wb, real n_l, real lnL, real dtc, U4 rnd)
+                                                     real wa, real wb, real n_l, real lnL, real dtc, Draw rnd)
 {
     if (qa == RF(0.0) || qb == RF(0.0)) return Collided{ua, ub, 0};
-    const real r0 = u01(rnd.x), r1 = u01(rnd.y), r2 = u01(rnd.z), r3 = u01(rnd.w);
     // divisions by the same quantity are done once, as a reciprocal
     const real ga = r_sqrt(r_fma(ua.z, ua.z, r_fma(ua.y, ua.y, r_fma(ua.x, ua.x, RF(1.0)))));
     const real gb = r_sqrt(r_fma(ub.z, ub.z, r_fma(ub.y, ub.y, r_fma(ub.x, ub.x, RF(1.0)))));
@@ -480,9 +506,9 @@ __device__ __forceinline__ Collided binary_collision(real4 ua, real4 ub, real ma
     const real q2 = r_mul(qa, qb);
     const real var = r_mul(r_mul(r_mul(r_mul(r_mul(k0, q2), q2), n_l), lnL), dtc) /
                      r_mul(r_mul(r_mul(r_mul(mu, mu), vrel), vrel), vrel);
-    const real delta = r_mul(r_mul(r_sqrt(var), r_sqrt(r_mul(-RF(2.0), r_log(r0)))), r_cospi(r_mul(RF(2.0), r1)));
-    real sphi, cphi;
-    r_sincospi(r_mul(RF(2.0), r2), &sphi, &cphi);
+    const CollDraw dr = coll_draw(rnd);
+    const real r3 = dr.r3, sphi = dr.sphi, cphi = dr.cphi;
+    const real delta = r_mul(r_mul(r_sqrt(var), dr.a), dr.c);
 
     const real pax = r_mul(ma, ua.x), pay = r_mul(ma, ua.y), paz = r_mul(ma, ua.z);
     const real Ea = r_mul(ma, ga), iE = RF(1.0) / r_fma(mb, gb, Ea);
