@@ -565,33 +565,131 @@ struct SeedArgs {
 
 __device__ __forceinline__ double u01d(uint32_t x) { return ((double)(x >> 9) + 0.5) * (1.0 / 8388608.0); }
 
+// momentum of particle i of the species: a beam electron's from draws 0 and
+// 1 of its stream, a Maxwellian one from draw 2
+__device__ __noinline__ void seed_momentum(const SeedArgs &a, const U4 &r0, const U4 &r1, const U4 &r2, bool beam,
+                                           double (&u)[3])
+{
+    if (beam) {
+        const double c = 2.0 * u01d(r0.w) - 1.0, ph = 2.0 * kPi * u01d(r1.x);
+        const double sn = sqrt(fmax(0.0, 1.0 - c * c));
+        u[0] = a.beam_u * sn * cos(ph); u[1] = a.beam_u * sn * sin(ph); u[2] = a.beam_u * c;
+    } else {
+        const double m1 = sqrt(-2.0 * log(u01d(r2.x))), t1 = 2.0 * kPi * u01d(r2.y);
+        const double m2 = sqrt(-2.0 * log(u01d(r2.z))), t2 = 2.0 * kPi * u01d(r2.w);
+        u[0] = a.sigma_u * m1 * cos(t1); u[1] = a.sigma_u * m1 * sin(t1); u[2] = a.sigma_u * m2 * cos(t2);
+    }
+}
+
+// log of the uniform of x, (2 k + 1) 2^-24 = m 2^e with m in [3/4, 3/2): from
+// a table {1 / c, log c} at c = 3/4 + j / 128 and the series of log(m / c),
+// |m / c - 1| <= 1/192, to the seventh power.  c = 1 for m near 1, where the
+// logarithm is small and the series alone; relative error below 2^-44.
+constexpr int SEED_LOG = 97;
+__device__ __forceinline__ double seed_log(uint32_t x, const double2 *tab)
+{
+    const uint32_t n = 2u * (x >> 9) + 1u;                     // 24 bits, odd
+    const int p = 31 - __clz(n);
+    const uint32_t frac = (n << (23 - p)) & 0x7fffffu;         // m = 1.frac, halved from 3/2 on
+    const uint32_t half = frac >> 22;
+    const double m = __hiloint2double((int)(((1023u - half) << 20) | (frac >> 3)), (int)(frac << 29));
+    const int j = (int)((__uint_as_float(((127u - half) << 23) | frac) - 0.75f) * 128.0f + 0.5f);
+    const double2 c = tab[j];
+    const double r = fma(m, c.x, -1.0);
+    double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
+    q = fma(r, q, 1.0 / 5.0);
+    q = fma(r, q, -1.0 / 4.0);
+    q = fma(r, q, 1.0 / 3.0);
+    q = fma(r, q, -1.0 / 2.0);
+    q = fma(r * r, q, r);
+    return fma((double)(p - 24 + (int)half), 0.6931471805599453, c.y + q);
+}
+
+// sine and cosine of t = 2 pi u, u the uniform of x: the quarter turn from
+// the integer, the rest of t (to 106 bits of pi/2) by the Taylor series to
+// the 15th and 16th power; relative error below 2^-50
+__device__ __forceinline__ void seed_sincos(double t, uint32_t x, double &sn, double &cs)
+{
+    const int n = (int)((4u * (x >> 9) + 2u + (1u << 22)) >> 23);
+    const double q = (double)n;
+    double r = fma(-q, 1.5707963267948966, t);
+    r = fma(-q, 6.123233995736766e-17, r);
+    const double z = r * r;
+    double s = fma(z, -1.0 / 1307674368000.0, 1.0 / 6227020800.0);
+    s = fma(z, s, -1.0 / 39916800.0);
+    s = fma(z, s, 1.0 / 362880.0);
+    s = fma(z, s, -1.0 / 5040.0);
+    s = fma(z, s, 1.0 / 120.0);
+    s = fma(z, s, -1.0 / 6.0);
+    s = fma(r * z, s, r);
+    double c = fma(z, 1.0 / 20922789888000.0, -1.0 / 87178291200.0);
+    c = fma(z, c, 1.0 / 479001600.0);
+    c = fma(z, c, -1.0 / 3628800.0);
+    c = fma(z, c, 1.0 / 40320.0);
+    c = fma(z, c, -1.0 / 720.0);
+    c = fma(z, c, 1.0 / 24.0);
+    c = fma(z, c, -1.0 / 2.0);
+    c = fma(z, c, 1.0);
+    const double a = n & 1 ? c : s, b = n & 1 ? s : c;
+    sn = n & 2 ? -a : a;
+    cs = (n + 1) & 2 ? -b : b;
+}
+
+// is v, known to 2^-40, surely on one side of the middle of the two floats
+// around it?
+__device__ __forceinline__ bool rounds_surely(double v)
+{
+    const int low = __double2loint(v) & 0x1fffffff;
+    return abs(low - 0x10000000) > 0x1000;
+}
+
+// The same momentum, for single-precision records: with the library's log,
+// sin, cos in double precision the seeding ran at the rate of the few double-
+// precision units (75 ms for 210 M particles, both species); with the forms
+// above, a third of their operations, it takes 44.  Where a component lies so near the middle of two
+// floats that their error could round it the other way (one in 2^16), the
+// particle is redone by seed_momentum: the records are the same bit for bit.
+__device__ __forceinline__ void seed_momentum_f32(const SeedArgs &a, const U4 &r0, const U4 &r1, const U4 &r2, bool beam,
+                                                  const double2 *tab, double (&u)[3])
+{
+    const double c = 2.0 * u01d(r0.w) - 1.0;
+    const uint32_t xa = beam ? r1.x : r2.y;
+    const double amp = (beam ? a.beam_u : a.sigma_u) * sqrt(beam ? fmax(0.0, 1.0 - c * c) : -2.0 * seed_log(r2.x, tab));
+    double sn, cs, s2, c2;
+    seed_sincos(2.0 * kPi * u01d(xa), xa, sn, cs);
+    seed_sincos(2.0 * kPi * u01d(r2.w), r2.w, s2, c2);
+    u[0] = amp * cs; u[1] = amp * sn;
+    u[2] = beam ? a.beam_u * c : a.sigma_u * sqrt(-2.0 * seed_log(r2.z, tab)) * c2;
+    if (!(rounds_surely(u[0]) && rounds_surely(u[1]) && (beam || rounds_surely(u[2])))) seed_momentum(a, r0, r1, r2, beam, u);
+}
+
 // particle i of the species: cell i / ppc (cell-major), id i; three draws of
 // its own stream give the position, the beam choice and direction, and two
 // Box-Muller pairs for the Maxwellian
-__global__ void k_seed(SeedArgs a)
+__global__ void __launch_bounds__(256) k_seed(SeedArgs a)
 {
+    __shared__ double2 tab[SEED_LOG];
+    for (int j = threadIdx.x; j < SEED_LOG; j += blockDim.x) {
+        const double c = 0.75 + j * (1.0 / 128.0);
+        tab[j] = make_double2(1.0 / c, log(c));
+    }
+    __syncthreads();
     const uint32_t pu = a.electrons ? PU_SEED_E : PU_SEED_I;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.n;
          i += (long long)gridDim.x * blockDim.x) {
         const int g = (int)(i / a.ppc);
         const U4 r0 = draw(a.seed, (unsigned long long)i, 0u, pu);
         const U4 r1 = draw(a.seed, (unsigned long long)i, 1u, pu);
+        const U4 r2 = draw(a.seed, (unsigned long long)i, 2u, pu);
         const real xi = u01(r0.x);
         const real eta = a.ny > 1 ? u01(r0.y) : RF(0.5);
-        double ux, uy, uz;
-        if (a.electrons && u01d(r0.z) < a.beam_frac) {
-            const double c = 2.0 * u01d(r0.w) - 1.0, ph = 2.0 * kPi * u01d(r1.x);
-            const double sn = sqrt(fmax(0.0, 1.0 - c * c));
-            ux = a.beam_u * sn * cos(ph); uy = a.beam_u * sn * sin(ph); uz = a.beam_u * c;
-        } else {
-            const U4 r2 = draw(a.seed, (unsigned long long)i, 2u, pu);
-            const double m1 = sqrt(-2.0 * log(u01d(r2.x))), t1 = 2.0 * kPi * u01d(r2.y);
-            const double m2 = sqrt(-2.0 * log(u01d(r2.z))), t2 = 2.0 * kPi * u01d(r2.w);
-            ux = a.sigma_u * m1 * cos(t1); uy = a.sigma_u * m1 * sin(t1); uz = a.sigma_u * m2 * cos(t2);
-        }
-        a.p0[i] = make_real4(xi, eta, (real)ux, (real)uy);
-        a.p1[i] = a.electrons ? rec_e1((real)uz, (real)a.w, (uint64_t)i)
-                              : rec_i1((real)uz, RF(0.0), (uint32_t)i, a.st);
+        const bool beam = a.electrons && u01d(r0.z) < a.beam_frac;
+        double u[3];
+        if constexpr (sizeof(real) == 4) seed_momentum_f32(a, r0, r1, r2, beam, tab, u);
+        else seed_momentum(a, r0, r1, r2, beam, u);
+        a.p0[i] = make_real4(xi, eta, (real)u[0], (real)u[1]);
+        a.p1[i] = a.electrons ? rec_e1((real)u[2], (real)a.w, (uint64_t)i)
+                              : rec_i1((real)u[2], RF(0.0), (uint32_t)i, a.st);
         a.key[i] = g;
     }
 }
