@@ -515,15 +515,15 @@ def _ion_args(st):
 
 def _electron_out(n, full=False):
     ft, ct = (np.float64, C.c_double) if full else (np.float32, C.c_float)
-    d = dict(X=np.zeros(n), Y=np.zeros(n), u=np.zeros((n, 3), dtype=ft), w=np.zeros(n, dtype=ft),
-             id=np.zeros(n, dtype=np.uint64))
+    d = dict(X=np.empty(n), Y=np.empty(n), u=np.empty((n, 3), dtype=ft), w=np.empty(n, dtype=ft),
+             id=np.empty(n, dtype=np.uint64))
     return d, (_p(d["X"]), _p(d["Y"]), _p(d["u"], ct), _p(d["w"], ct), _p(d["id"], C.c_uint64))
 
 
 def _ion_out(n, full=False):
     ft, ct = (np.float64, C.c_double) if full else (np.float32, C.c_float)
-    d = dict(X=np.zeros(n), Y=np.zeros(n), u=np.zeros((n, 3), dtype=ft), zf=np.zeros(n, dtype=ft),
-             Z=np.zeros(n, dtype=np.int32), nK=np.zeros(n, dtype=np.int32), id=np.zeros(n, dtype=np.uint32))
+    d = dict(X=np.empty(n), Y=np.empty(n), u=np.empty((n, 3), dtype=ft), zf=np.empty(n, dtype=ft),
+             Z=np.empty(n, dtype=np.int32), nK=np.empty(n, dtype=np.int32), id=np.empty(n, dtype=np.uint32))
     return d, (_p(d["X"]), _p(d["Y"]), _p(d["u"], ct), _p(d["zf"], ct), _p(d["Z"], C.c_int32),
                _p(d["nK"], C.c_int32), _p(d["id"], C.c_uint32))
 

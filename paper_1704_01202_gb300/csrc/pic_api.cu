@@ -15,6 +15,7 @@
 #include <cstddef>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -58,6 +59,26 @@ int next_pow2(int x)
     return p;
 }
 
+// host records without the zeroing of a vector (every one is written)
+template <class T>
+struct HostBuf {
+    std::unique_ptr<T[]> p;
+    size_t n = 0;
+    void resize(size_t m)
+    {
+        p.reset(m ? new T[m] : nullptr);
+        n = m;
+    }
+    size_t size() const { return n; }
+    T *data() { return p.get(); }
+    const T *data() const { return p.get(); }
+    T &operator[](size_t k) { return p[k]; }
+    const T &operator[](size_t k) const { return p[k]; }
+};
+
+typedef HostBuf<real4> HostRecs;
+typedef HostBuf<int> HostKeys;
+
 }  // namespace
 
 struct pic_ctx {
@@ -74,8 +95,8 @@ struct pic_ctx {
     std::vector<pic_grid> grids;         // grid of each slot as given
     struct Pending {                     // admitted, particles not yet on the device
         int slot;
-        std::vector<real4> e0, e1, i0, i1;
-        std::vector<int> ek, ik;
+        HostRecs e0, e1, i0, i1;
+        HostKeys ek, ik;
     };
     std::vector<Pending> pending;
     int ncell = 0, npts = 0, nblk = 0, nrows = 0, max_row_nx = 0;
@@ -968,8 +989,8 @@ pic_status ctx_create(pic_ctx **out, int nslot, int slot_cells, int slot_pts, in
 // (xi, eta, ux, uy), (uz, w | zfrac, id, state) and the global cell key.
 pic_status build_records(pic_ctx *c, int slot, const pic_grid *g, bool electrons, int64_t n, const double *X,
                          const double *Y, const float *u, const float *w_or_zf, const uint64_t *eid,
-                         const int32_t *Z, const int32_t *nK, const uint32_t *iid, std::vector<real4> &p0,
-                         std::vector<real4> &p1, std::vector<int> &key)
+                         const int32_t *Z, const int32_t *nK, const uint32_t *iid, HostRecs &p0,
+                         HostRecs &p1, HostKeys &key)
 {
     p0.resize(n); p1.resize(n); key.resize(n);
     const int cell0 = slot * c->slot_cells;
@@ -997,8 +1018,8 @@ pic_status build_records(pic_ctx *c, int slot, const pic_grid *g, bool electrons
         }
         return 0;
     };
-    // large loads are split over host threads (disjoint ranges, same records)
-    const int64_t per = 1 << 20;
+    // larger loads are split over host threads (disjoint ranges, same records)
+    const int64_t per = 1 << 16;
     const int nt = (int)std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), (n + per - 1) / per);
     std::vector<int> rc(std::max(nt, 1), 0);
     if (nt <= 1) {
@@ -1042,8 +1063,8 @@ pic_status sort_species(pic_ctx *c, bool electrons, int64_t n)
     return PIC_OK;
 }
 
-pic_status load_species(pic_ctx *c, bool electrons, int64_t n, const std::vector<real4> &p0,
-                        const std::vector<real4> &p1, const std::vector<int> &key)
+pic_status load_species(pic_ctx *c, bool electrons, int64_t n, const HostRecs &p0, const HostRecs &p1,
+                        const HostKeys &key)
 {
     cudaStream_t st = c->stream;
     if (n > 0) {
@@ -1057,9 +1078,7 @@ pic_status load_species(pic_ctx *c, bool electrons, int64_t n, const std::vector
 // Admission: host records are appended behind the sorted particles of each
 // species, every sorted particle is keyed by its own cell (-1 when its slab
 // is inactive), and one count / scan / scatter re-sorts all of them.
-pic_status resort_with(pic_ctx *c, const std::vector<real4> &e0, const std::vector<real4> &e1,
-                       const std::vector<int> &ek, const std::vector<real4> &i0, const std::vector<real4> &i1,
-                       const std::vector<int> &ik)
+pic_status resort_with(pic_ctx *c, const std::vector<pic_ctx::Pending> &add)
 {
     cudaStream_t st = c->stream;
     int ns[2] = {0, 0};
@@ -1069,21 +1088,25 @@ pic_status resort_with(pic_ctx *c, const std::vector<real4> &e0, const std::vect
     const int nxt = c->cur ^ 1;
     for (int sp = 0; sp < 2; ++sp) {
         const bool el = sp == 0;
-        const std::vector<real4> &h0 = el ? e0 : i0, &h1 = el ? e1 : i1;
-        const std::vector<int> &hk = el ? ek : ik;
-        const long long n0 = ns[sp], nadd = (long long)hk.size();
+        long long n0 = ns[sp], nadd = 0;
+        for (const auto &p : add) nadd += (long long)(el ? p.ek : p.ik).size();
         if (n0 + nadd > (el ? c->cap_e : c->cap_i))
             return fail(c, PIC_ERR_CAPACITY, "particle capacity exceeded by admission");
         real4 *A0 = el ? c->eA0 : c->iA0, *A1 = el ? c->eA1 : c->iA1, *B0 = el ? c->eB0 : c->iB0, *B1 = el ? c->eB1 : c->iB1;
         int *key = el ? c->ekey : c->ikey, *cnt = el ? c->cnt_e : c->cnt_i, *fill = el ? c->fill_e : c->fill_i;
         const int *cs = el ? c->csE[c->cur] : c->csI[c->cur];
         k_cell_keys<<<c->nsm * 4, 256, 0, st>>>(cs, c->ncell, c->cell_slab, c->d_slab, key);
-        if (nadd) {
-            CK(cudaMemcpyAsync(A0 + n0, h0.data(), sizeof(real4) * nadd, cudaMemcpyHostToDevice, st));
-            CK(cudaMemcpyAsync(A1 + n0, h1.data(), sizeof(real4) * nadd, cudaMemcpyHostToDevice, st));
-            CK(cudaMemcpyAsync(key + n0, hk.data(), sizeof(int) * nadd, cudaMemcpyHostToDevice, st));
-        }
         const int tot = (int)(n0 + nadd);
+        for (const auto &p : add) {
+            const HostRecs &h0 = el ? p.e0 : p.i0, &h1 = el ? p.e1 : p.i1;
+            const HostKeys &hk = el ? p.ek : p.ik;
+            const size_t m = hk.size();
+            if (!m) continue;
+            CK(cudaMemcpyAsync(A0 + n0, h0.data(), sizeof(real4) * m, cudaMemcpyHostToDevice, st));
+            CK(cudaMemcpyAsync(A1 + n0, h1.data(), sizeof(real4) * m, cudaMemcpyHostToDevice, st));
+            CK(cudaMemcpyAsync(key + n0, hk.data(), sizeof(int) * m, cudaMemcpyHostToDevice, st));
+            n0 += (long long)m;
+        }
         CK(cudaMemcpyAsync(c->counters + CNT_NLOAD, &tot, sizeof(int), cudaMemcpyHostToDevice, st));
         CK(cudaMemsetAsync(cnt, 0, sizeof(int) * c->ncell, st));
         CK(cudaMemsetAsync(fill, 0, sizeof(int) * c->ncell, st));
@@ -1105,9 +1128,7 @@ pic_status resort_with(pic_ctx *c, const std::vector<real4> &e0, const std::vect
 // drop the particles of retired slabs now (one re-sort) and free their slots
 pic_status compact(pic_ctx *c)
 {
-    const std::vector<real4> no4;
-    const std::vector<int> noi;
-    pic_status r = resort_with(c, no4, no4, noi, no4, no4, noi);
+    pic_status r = resort_with(c, {});
     if (r != PIC_OK) return r;
     for (int k = 0; k < c->nslot; ++k)
         if (c->slot_state[k] == 2) c->slot_state[k] = 0;
@@ -1138,23 +1159,20 @@ pic_status apply_pending(pic_ctx *c)
             if (r != PIC_OK) return r;
         }
     }
-    std::vector<real4> e0, e1, i0, i1;
-    std::vector<int> ek, ik;
-    for (auto &p : c->pending) {
+    // the records go to the device from where they are: joining them first
+    // cost as much as forming them
+    for (const auto &p : c->pending) {
         c->slabs[p.slot].active = 1;
         pic_status r = reset_slot(c, p.slot);
         if (r != PIC_OK) return r;
-        e0.insert(e0.end(), p.e0.begin(), p.e0.end()); e1.insert(e1.end(), p.e1.begin(), p.e1.end());
-        ek.insert(ek.end(), p.ek.begin(), p.ek.end());
-        i0.insert(i0.end(), p.i0.begin(), p.i0.end()); i1.insert(i1.end(), p.i1.begin(), p.i1.end());
-        ik.insert(ik.end(), p.ik.begin(), p.ik.end());
     }
+    const std::vector<pic_ctx::Pending> add = std::move(c->pending);
     c->pending.clear();
-    return resort_with(c, e0, e1, ek, i0, i1, ik);
+    return resort_with(c, add);
 }
 
 // particles of one slot back on the host with the slot's cell starts
-pic_status fetch_slot(pic_ctx *c, int slot, bool electrons, std::vector<real4> &p0, std::vector<real4> &p1,
+pic_status fetch_slot(pic_ctx *c, int slot, bool electrons, HostRecs &p0, HostRecs &p1,
                       std::vector<int> &cs)
 {
     cudaStream_t st = c->stream;
@@ -1191,7 +1209,7 @@ pic_status counts_slot(pic_ctx *c, int slot, int64_t *n_e, int64_t *n_i)
 template <class U>
 pic_status get_electrons_slot(pic_ctx *c, int slot, double *X, double *Y, U *u, U *w, uint64_t *id)
 {
-    std::vector<real4> p0, p1;
+    HostRecs p0, p1;
     std::vector<int> cs;
     pic_status r = fetch_slot(c, slot, true, p0, p1, cs);
     if (r != PIC_OK) return r;
@@ -1213,7 +1231,7 @@ template <class U>
 pic_status get_ions_slot(pic_ctx *c, int slot, double *X, double *Y, U *u, U *zfrac, int32_t *Z,
                          int32_t *nK, uint32_t *id)
 {
-    std::vector<real4> p0, p1;
+    HostRecs p0, p1;
     std::vector<int> cs;
     pic_status r = fetch_slot(c, slot, false, p0, p1, cs);
     if (r != PIC_OK) return r;
@@ -1550,8 +1568,8 @@ pic_status pic_load_electrons(pic_ctx *c, int64_t n, const double *X, const doub
     if (!c || n < 0 || (n > 0 && (!X || !Y || !u || !w || !id))) return PIC_ERR_ARG;
     if (c->batch) return fail(c, PIC_ERR_STATE, "a batch context loads particles at admission");
     if (n > c->cap_e) return fail(c, PIC_ERR_CAPACITY, "more electrons than the capacity");
-    std::vector<real4> p0, p1;
-    std::vector<int> key;
+    HostRecs p0, p1;
+    HostKeys key;
     pic_status r = build_records(c, 0, &c->grids[0], true, n, X, Y, u, w, id, nullptr, nullptr, nullptr, p0, p1, key);
     if (r == PIC_OK) r = load_species(c, true, n, p0, p1, key);
     if (r == PIC_OK) c->loaded_e = true;
@@ -1596,8 +1614,8 @@ pic_status pic_load_ions(pic_ctx *c, int64_t n, const double *X, const double *Y
     if (!c || n < 0 || (n > 0 && (!X || !Y || !u || !zfrac || !Z || !nK || !id))) return PIC_ERR_ARG;
     if (c->batch) return fail(c, PIC_ERR_STATE, "a batch context loads particles at admission");
     if (n > c->cap_i) return fail(c, PIC_ERR_CAPACITY, "more ions than the capacity");
-    std::vector<real4> p0, p1;
-    std::vector<int> key;
+    HostRecs p0, p1;
+    HostKeys key;
     pic_status r = build_records(c, 0, &c->grids[0], false, n, X, Y, u, zfrac, nullptr, Z, nK, id, p0, p1, key);
     if (r == PIC_OK) r = load_species(c, false, n, p0, p1, key);
     if (r == PIC_OK) c->loaded_i = true;
@@ -2231,7 +2249,8 @@ pic_status pic_restore(pic_ctx *c, const void *host, size_t bytes)
     if (h.n_e > c->cap_e || h.n_i > c->cap_i) return fail(c, PIC_ERR_CAPACITY, "checkpoint exceeds the capacity");
     const char *p = (const char *)host + sizeof(CkptHeader);
     const int64_t ne = h.n_e, ni = h.n_i;
-    std::vector<real4> e0(ne), e1(ne), i0(ni), i1(ni);
+    HostRecs e0, e1, i0, i1;
+    e0.resize(ne); e1.resize(ne); i0.resize(ni); i1.resize(ni);
     std::vector<int> cse(c->ncell + 1), csi(c->ncell + 1);
     auto take = [&](void *dst, size_t n) { std::memcpy(dst, p, n); p += n; };
     take(e0.data(), sizeof(real4) * ne); take(e1.data(), sizeof(real4) * ne);
@@ -2251,7 +2270,8 @@ pic_status pic_restore(pic_ctx *c, const void *host, size_t bytes)
             !(i1[k].y >= (real)0 && i1[k].y < (real)1))
             return fail(c, PIC_ERR_ARG, "checkpoint ion record out of range");
     }
-    std::vector<int> ke(ne), ki(ni);
+    HostKeys ke, ki;
+    ke.resize(ne); ki.resize(ni);
     for (int g2 = 0; g2 < c->ncell; ++g2) {
         if (cse[g2 + 1] < cse[g2] || csi[g2 + 1] < csi[g2]) return fail(c, PIC_ERR_ARG, "checkpoint cell starts inconsistent");
         for (int k = cse[g2]; k < cse[g2 + 1]; ++k) ke[k] = g2;
