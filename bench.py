@@ -49,16 +49,16 @@ CELL_BYTES_PER_PARTICLE = 64
 # whole step: cell kernel 64 B + scatter (36 B read, 32 B written)
 STEP_BYTES_PER_PARTICLE = 132
 # DRAM bytes per particle of the cell kernel, from one ncu capture of a
-# smaller slab of the same make-up (1024 x 256 cells, 28.0 M particles:
-# 1782.5 MB on a plain step, 1829.6 MB on a radiation step, 64.0 B per
+# smaller slab of the same make-up (1024 x 256 cells, 26.4 M particles:
+# 1669.6 MB on a plain step, 1676.6 MB on a radiation step, 63.3 B per
 # particle over the five-step cycle), scaled to a launch by the particle
 # count; None when no capture of the current kernel exists
-CELL_TRAFFIC_BYTES_PER_PARTICLE = 64.0
+CELL_TRAFFIC_BYTES_PER_PARTICLE = 63.3
 # warp instructions per particle of the cell kernel, from the same capture
-# (104 on a radiation step, 89 on the others: 92 over the five-step cycle);
+# (76 on a radiation step, 61 on the others: 64 over the five-step cycle);
 # the kernel is bound by instruction issue, so the bench also sets its
 # time against the SM issue rate
-CELL_WARP_INSTR_PER_PARTICLE = 92.0
+CELL_WARP_INSTR_PER_PARTICLE = 64.2
 
 
 def measured_peaks():
@@ -194,16 +194,17 @@ def run_reference(args):
     print(json.dumps(out))
 
 
-def issue_rate(cell_ms, n_particles, n_sm, sm_mhz):
+def issue_rate(cell_ms, n_particles, n_sm, sm_mhz, per_particle=92.0):
     """The cell kernel against the SM issue rate: warp instructions per
     particle x particles over its time, against four schedulers per SM
     issuing one warp instruction a cycle at the SM clock sampled during the
-    timed steps (the maximum clock when no sample exists)."""
+    timed steps (the maximum clock when no sample exists).  `per_particle`
+    is the captured kernel's; the default is an earlier capture's."""
     mhz = sm_mhz if sm_mhz else 2070.0
     peak = 4.0 * n_sm * mhz * 1e6
-    achieved = CELL_WARP_INSTR_PER_PARTICLE * n_particles / (cell_ms * 1e-3)
+    achieved = per_particle * n_particles / (cell_ms * 1e-3)
     return {"achieved": achieved, "peak": peak, "unit": "warp instructions/s", "frac": achieved / peak,
-            "warp_instructions_per_particle": CELL_WARP_INSTR_PER_PARTICLE, "sm": n_sm, "sm_mhz": mhz,
+            "warp_instructions_per_particle": per_particle, "sm": n_sm, "sm_mhz": mhz,
             "source": "instructions per particle from ncu (profiles/)"}
 
 
@@ -345,7 +346,7 @@ def run_gpu(args):
             "kernel": "k_cell", "peak_source": peak_kind,
             "bytes_per_particle": CELL_BYTES_PER_PARTICLE, "kernel_ms_per_step": cell_ms,
             "share_of_step": tms["cell"] / max(tms["step"], 1e-9),
-            "issue": issue_rate(cell_ms, n_mean, n_sm, clk.get("sm_mhz"))}
+            "issue": issue_rate(cell_ms, n_mean, n_sm, clk.get("sm_mhz"), CELL_WARP_INSTR_PER_PARTICLE)}
     step_gbs = STEP_BYTES_PER_PARTICLE * n_mean / (ms / args.steps * 1e-3) / 1e9
 
     # end to end through the public API with host buffers

@@ -40,7 +40,7 @@ constexpr int CNT_APPEND = 0, CNT_WORK = 1, CNT_WORK_T1 = 2, CNT_WORK_BIG = 3, C
 // (k_begin clears [0, CNT_STEP_ZERO) and [CNT_MAXE, NCOUNTERS), 16-byte aligned)
 static_assert(CNT_MAXE % 4 == 0, "alignment of the cleared counters");
 constexpr int NEV = 6;   // timing events per step
-// largest cell of the one-warp pass (the FP64 build's staging is twice as
+// largest cell of the large-cell pass (the FP64 build's staging is twice as
 // wide and takes half the populations into the same shared memory)
 constexpr int BIG_CE = sizeof(real) == 8 ? 1024 : 2048, BIG_CI = sizeof(real) == 8 ? 256 : 512;
 
@@ -124,7 +124,7 @@ struct pic_ctx {
 
     // cell-kernel tiers: tier 0 takes every cell with the staging sizes
     // below; cells that do not fit go to tier 1 (sized for the largest
-    // cells, when that is larger), then to the one-warp large-cell pass
+    // cells, when that is larger), then to the large-cell pass
     int cap_ce = 128, cap_ci = 32, cap_new = 96, wpc = 4;
     int t1_ce = 0, t1_ci = 0, t1_wpc = 1;    // t1_ce == 0: no tier 1
     int t2_ce = 0, t2_ci = 0, t2_wpc = 1;    // t2_ce == 0: no tier 2
@@ -203,7 +203,7 @@ T *carve_arena(pic_ctx *c, size_t count)
 
 // Created-electron scratch of the cell launches, in entries: cap_new = 3 x
 // the ions a tier stages (at most 768 below the large-cell pass, whose
-// 1536 take one warp a CTA) for every warp resident at once, at most 16 a
+// 1536 take one team a CTA) for every warp resident at once, at most 16 a
 // SM (the register-bound instances) on up to 192 SMs, and no more warps
 // than cells (plus a CTA).  Launch grids are clamped to the slices.
 // Contexts of up to WHOLE_CELLS cells (and two an SM: that staging is 100 KB)
@@ -1454,7 +1454,7 @@ pic_status read_budget_failures(pic_ctx *c)
 
 // Steps between two re-sizings of the cell tiers inside one pic_step call:
 // ionization grows the cells, and cells that outgrow the tiers fall through
-// to the one-warp large-cell pass.  Even, so that step pairs replay whole.
+// to the large-cell pass.  Even, so that step pairs replay whole.
 constexpr int RESIZE_EVERY = 32;
 
 pic_status step_chunk(pic_ctx *c, int n);
