@@ -698,9 +698,11 @@ pic_status launch_step(pic_ctx *c)
     ++c->launches;
     if (ev) CK(cudaEventRecord(ev[4], st));
     const AdvanceArgs adv{c->d_steps, c->d_slab, c->nslot, c->slab_app, c->slab_err};
+    const int nsub = shape.nsub;
+    // narrow 1D slots: a block each does the update and the step end (k_field_1d)
+    const bool field_1d = c->slot_rows == 1 && nsub == 1 && c->slot_pts <= FIELD1_PTS;
     if (shape.field) {
         nv.phase("fields");
-        const int nsub = shape.nsub;
         FieldArgs f{};
         f.slabs = c->d_slab; f.pt_slab = c->pt_slab; f.npts = c->npts; f.B = c->B; f.J = c->J;
         int fg = std::min((c->npts + 255) / 256, c->nsm * 16);
@@ -709,7 +711,7 @@ pic_status launch_step(pic_ctx *c)
             f.Ein = c->E[c->ecur]; f.Eout = c->E[c->ecur ^ 1];
             c->ecur ^= 1;
             const bool last = sub == nsub - 1;
-            if (c->slot_rows == 1 && nsub == 1) {
+            if (field_1d) {
                 k_field_1d<<<c->nslot, FIELD1_T, 0, st>>>(f, adv, c->slot_pts);
                 ++c->launches;
                 continue;
@@ -722,7 +724,7 @@ pic_status launch_step(pic_ctx *c)
             c->launches += 3;
         }
     }
-    if (!shape.field || (c->batch && shape.nsub > 1)) {
+    if (!shape.field || (c->batch && !field_1d)) {
         k_advance<<<(c->nslot + 127) / 128, 128, 0, st>>>(adv);
         ++c->launches;
     }

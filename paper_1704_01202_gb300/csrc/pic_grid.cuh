@@ -418,12 +418,18 @@ __global__ void k_b_half_advance(FieldArgs a, AdvanceArgs v)
 }
 
 // The field update of 1D slabs, a block each (slot_pts grid points), and the
-// end of their step.  A slab's update is a few hundred points three times
-// over; as four launches it took 21 us of a small slab's step, most of it
-// starting and ending, as one 9 (128 cells; 24 slabs of 250 cells 21 -> 11,
-// 20 of up to 2048, 25 -> 26: a block's three passes there cost what the
-// launches did).
-constexpr int FIELD1_T = 512;
+// end of their step.  A narrow slab's update is a few hundred points three
+// times over: as three or four launches most of its 17-23 us are their starts
+// and ends, as one it takes 8.5 (128 cells).  But the block's passes grow with
+// the width (33 us at 4096 cells, 66 at 8192, one SM busy), while the launches over
+// all points stay at 17-25 us, so wider slots take those.  Measured per step
+// by graph replay (push and fields, 3 particles a cell), one block a slab |
+// grid-wide: alone 128 cells 27.8 | 31.7 us, 512 34.6 | 36.6, 768 38.4 | 38.5,
+// 1024 40.3 | 39.6, 2048 51.9 | 45.6, 8192 125 | 74; 24 slabs of 512 99.0 |
+// 102.8, 1024 161.9 | 161.9, 2048 294 | 288, 8192 1023 | 971; 96 of 1024 537 |
+// 536; 256 of 512 703.6 | 704.5, 1024 1393 | 1392, 4096 5634 | 5625.  The two
+// meet at 768 to 1024 cells whatever the number of slabs.
+constexpr int FIELD1_T = 512, FIELD1_PTS = 1024;
 __global__ void __launch_bounds__(FIELD1_T) k_field_1d(FieldArgs a, AdvanceArgs v, int slot_pts)
 {
     const int s = blockIdx.x, p0 = s * slot_pts;
