@@ -283,7 +283,7 @@ def run_gpu(args):
     # steps autotune the cell kernel's launch shape for the state the timed
     # steps see (these are real steps of the run)
     n_adv = int(round(args.advance_fs / cfg.dt_fs))
-    tune_steps = 0 if args.no_autotune else min(9, n_adv)
+    tune_steps = 0 if args.no_autotune else min(10, n_adv)
     adv = {"steps": n_adv, "fs": n_adv * cfg.dt_fs}
     ne_a, ni_a = slab.counts()
     d_start = slab.diagnostics()
@@ -409,7 +409,7 @@ def run_rt(pkg, tab, args):
     slab.set_rt(coarsen=8, n_polar=4, n_azimuth=2, scheme=0)
     stream = torch.cuda.current_stream()
     slab.autotune(True)
-    slab.step(9)
+    slab.step(10)
     slab.autotune(False)
     slab.step(max(args.warmup, 3))
     slab.sync()
@@ -447,7 +447,7 @@ def run_foil(pkg, tab, args):
     del st
     stream = torch.cuda.current_stream()
     slab.autotune(True)
-    slab.step(9)
+    slab.step(10)
     slab.autotune(False)
     slab.step(max(args.warmup, 3))
     slab.sync()
@@ -506,7 +506,7 @@ def run_ensemble(pkg, tab, args, rank):
     for (c, pl), st in zip(ens, states):
         bt.admit(c, st, pl)
     bt.autotune(True)
-    bt.step(9 + args.warmup)
+    bt.step(10 + args.warmup)
     bt.autotune(False)
     bt.sync()
     tuned = bt.autotune()

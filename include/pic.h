@@ -413,8 +413,9 @@ pic_status pic_use_graphs(pic_ctx *c, int enable);
  * steps run the cell kernel with 1, 2, 4 and 8 warps per CTA (as many as fit
  * in shared memory; 4 alone where a cell takes a team of four), each twice
  * in the order 1 2 4 8 8 4 2 1, timing the cell kernels with CUDA events; the
- * fastest mean is kept for those sizes.
- * The context's first step is not timed.  These are steps of the
+ * fastest mean is kept for those sizes.  The context's first step is not
+ * timed, nor are steps on which a slab has radiation, unless all are such
+ * (with one in five, 8 times take at most 10 steps).  These are steps of the
  * simulation: the launch shape changes no result.  enable = 0 stops tuning
  * (choices made are kept); -1 leaves it as is.  wpc_out (may be NULL) gets
  * the warps per CTA in use; ms_out (4 floats, may be NULL) the mean cell
