@@ -26,6 +26,7 @@
 #include "pic_cellk.cuh"
 #include "pic_push.cuh"
 #include "pic_grid.cuh"
+#include "pic_host.cuh"
 #include "pic_rt.cuh"
 
 using namespace pic;
@@ -1024,14 +1025,7 @@ pic_status build_records(pic_ctx *c, int slot, const pic_grid *g, bool electrons
     const int64_t per = 1 << 16;
     const int nt = (int)std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), (n + per - 1) / per);
     std::vector<int> rc(std::max(nt, 1), 0);
-    if (nt <= 1) {
-        rc[0] = fill(0, n);
-    } else {
-        std::vector<std::thread> th;
-        for (int t = 0; t < nt; ++t)
-            th.emplace_back([&, t] { rc[t] = fill(n * t / nt, n * (t + 1) / nt); });
-        for (auto &x : th) x.join();
-    }
+    host_shares(nt, [&](int t) { rc[t] = fill(n * t / nt, n * (t + 1) / nt); });
     for (int r : rc) {
         if (r == 1) return fail(c, PIC_ERR_ARG, "particle position outside the slab");
         if (r == 2) return fail(c, PIC_ERR_ARG, "ion state out of range");
