@@ -202,16 +202,19 @@ T *carve_arena(pic_ctx *c, size_t count)
     return p;
 }
 
+// Contexts of up to WHOLE_CELLS cells (and two an SM: that staging is 100 KB;
+// 304 on the 152 SMs of a GB300) stage every cell at the large-cell pass's
+// size: no pass for what outgrows its tier, and nothing to re-size between
+// steps.  257 cells of 123 electrons and 31 ions, a step: 94 -> 57 us with the
+// one-launch field update.
+constexpr int WHOLE_CELLS = 304;
+
 // Created-electron scratch of the cell launches, in entries: cap_new = 3 x
 // the ions a tier stages (at most 768 below the large-cell pass, whose
 // 1536 take one team a CTA) for every warp resident at once, at most 16 a
 // SM (the register-bound instances) on up to 192 SMs, and no more warps
-// than cells (plus a CTA).  Launch grids are clamped to the slices.
-// Contexts of up to WHOLE_CELLS cells (and two an SM: that staging is 100 KB)
-// stage every cell at the large-cell pass's size: no pass for what outgrows
-// its tier, and nothing to re-size between steps.  257 cells of 123 electrons
-// and 31 ions, a step: 94 -> 57 us with the one-launch field update.
-constexpr int WHOLE_CELLS = 384;
+// than cells (plus a CTA); 1536 for every team of the contexts above.
+// Launch grids are clamped to the slices.
 size_t nw_scratch_entries(int ncell)
 {
     const size_t warps = std::min<size_t>(192 * 16, (size_t)ncell + 64);
