@@ -41,6 +41,11 @@ struct PushArgs {
 // (the FP64 build halves the warps per CTA: its rows are twice as wide)
 constexpr int PUSH_TEAM = 4, PUSH_NEW_CTAS = 64;
 constexpr int JROWS = 40, JPITCH = 36, PUSH_WARPS = sizeof(real) == 8 ? 4 : 8;
+struct __align__(kSmAlign) JStage { real v[JROWS * JPITCH]; };
+// jrows reads the rows as real4 (32-byte aligned in the FP64 build)
+static_assert(alignof(JStage) >= alignof(real4) && JPITCH * sizeof(real) % alignof(real4) == 0 &&
+                  sizeof(JStage) % alignof(real4) == 0,
+              "alignment of the stencil rows");
 
 __device__ __forceinline__ void jput(real *col, int k, real v) { col[k * JPITCH] = v; }
 
@@ -505,11 +510,11 @@ __device__ __forceinline__ void push_created(const PushArgs &a, int t0, int nt)
 template <int DIM>
 __global__ void __launch_bounds__(32 * PUSH_WARPS, DIM == 2 ? 5 : 2) k_push(PushArgs a)
 {
-    __shared__ __align__(16) real s_j[PUSH_WARPS][JROWS * JPITCH];
+    __shared__ JStage s_j[PUSH_WARPS];
     __shared__ real s_t[PUSH_WARPS][TILE];
     __shared__ PushSlab s_slab[PUSH_WARPS];
     const int lane = threadIdx.x & 31;
-    real *sj = s_j[threadIdx.x >> 5];
+    real *sj = s_j[threadIdx.x >> 5].v;
     real *tile = s_t[threadIdx.x >> 5];
     PushSlab &S = s_slab[threadIdx.x >> 5];
     push_created(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
@@ -545,7 +550,7 @@ __global__ void __launch_bounds__(32 * PUSH_WARPS, DIM == 2 ? 5 : 2) k_push(Push
 template <int DIM, int TW>
 __global__ void __launch_bounds__(32 * TW, 4) k_push_team(PushArgs a)
 {
-    __shared__ __align__(16) real s_j[TW][JROWS * JPITCH];
+    __shared__ JStage s_j[TW];
     __shared__ real s_t[TILE], s_tot[2 * TW * JROWS];
     __shared__ PushSlab S;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = (int)blockIdx.x - PUSH_NEW_CTAS;
@@ -562,7 +567,7 @@ __global__ void __launch_bounds__(32 * TW, 4) k_push_team(PushArgs a)
         for (int k = i0 + threadIdx.x; k < i1; k += 32 * TW) a.ikey[k] = -1;
         return;
     }
-    push_cell<DIM, TW>(a, S, g, warp, lane, s_j[warp], s_t, s_tot);
+    push_cell<DIM, TW>(a, S, g, warp, lane, s_j[warp].v, s_t, s_tot);
 }
 
 }  // namespace pic
