@@ -1028,7 +1028,10 @@ pic_status build_records(pic_ctx *c, int slot, const pic_grid *g, bool electrons
     const int64_t per = 1 << 16;
     const int nt = (int)std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()), (n + per - 1) / per);
     std::vector<int> rc(std::max(nt, 1), 0);
-    host_shares(nt, [&](int t) { rc[t] = fill(n * t / nt, n * (t + 1) / nt); });
+    // (called through the shares' function, a small load's loop is a tenth
+    // slower: 24 slabs of 20,000 particles 4.4 -> 4.8 ms)
+    if (nt <= 1) rc[0] = fill(0, n);
+    else host_shares(nt, [&](int t) { rc[t] = fill(n * t / nt, n * (t + 1) / nt); });
     for (int r : rc) {
         if (r == 1) return fail(c, PIC_ERR_ARG, "particle position outside the slab");
         if (r == 2) return fail(c, PIC_ERR_ARG, "ion state out of range");
