@@ -199,7 +199,9 @@ def issue_rate(cell_ms, n_particles, n_sm, sm_mhz, per_particle=92.0):
     particle x particles over its time, against four schedulers per SM
     issuing one warp instruction a cycle at the SM clock sampled during the
     timed steps (the maximum clock when no sample exists).  `per_particle`
-    is the captured kernel's; the default is an earlier capture's."""
+    is the captured kernel's (the bench passes the current capture's; the
+    default is that of an earlier kernel, which a test of this arithmetic
+    takes)."""
     mhz = sm_mhz if sm_mhz else 2070.0
     peak = 4.0 * n_sm * mhz * 1e6
     achieved = per_particle * n_particles / (cell_ms * 1e-3)

@@ -501,12 +501,15 @@ __device__ __forceinline__ void push_created(const PushArgs &a, int t0, int nt)
 
 // One warp per cell, cells handed out from a counter.  Bound by the latency
 // of dependent loads and arithmetic (14 % of DRAM throughput at 16 warps an
-// SM), so 2D runs five CTAs an SM (48 registers); in 1D, with a quarter of
-// the stencil's arithmetic, two CTAs without spills are faster.  2048 x 256
+// SM).  The stencil rows are 48 KB a CTA, so four are resident, 32 warps an SM:
+// the bound of five in 2D is there for its register cap (48).  2048 x 256
 // cells, 42 M particles, a step: 2.90 ms with scalar reads of the stencil
 // rows, all 40 weights formed from four-node shapes and 16 warps an SM; 1.82
 // ms with 16-byte row reads, the weights that are zero left out, the next
-// cell's records prefetched and 40 warps an SM (2.00 ms at 32, 1.86 at 48).
+// cell's records prefetched and four CTAs an SM at 48 registers, spills included
+// (64 registers, the bound of four: 2.00 ms; 40, the bound of six: 1.86).
+// In 1D, with a quarter of the stencil's arithmetic, two CTAs without spills
+// are faster.
 template <int DIM>
 __global__ void __launch_bounds__(32 * PUSH_WARPS, DIM == 2 ? 5 : 2) k_push(PushArgs a)
 {
