@@ -2315,11 +2315,8 @@ pic_status pic_restore(pic_ctx *c, const void *host, size_t bytes)
     }
     HostKeys ke, ki;
     ke.resize(ne); ki.resize(ni);
-    for (int g2 = 0; g2 < c->ncell; ++g2) {
-        if (cse[g2 + 1] < cse[g2] || csi[g2 + 1] < csi[g2]) return fail(c, PIC_ERR_ARG, "checkpoint cell starts inconsistent");
-        for (int k = cse[g2]; k < cse[g2 + 1]; ++k) ke[k] = g2;
-        for (int k = csi[g2]; k < csi[g2 + 1]; ++k) ki[k] = g2;
-    }
+    if (!keys_of_starts(cse.data(), c->ncell, ne, ke.data()) || !keys_of_starts(csi.data(), c->ncell, ni, ki.data()))
+        return fail(c, PIC_ERR_ARG, "checkpoint cell starts inconsistent");
     pic_status r = load_species(c, true, ne, e0, e1, ke);
     if (r == PIC_OK) r = load_species(c, false, ni, i0, i1, ki);
     if (r != PIC_OK) return r;

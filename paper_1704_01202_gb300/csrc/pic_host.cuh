@@ -1,5 +1,6 @@
 // Host helpers of the C ABI (plain C++).
 #pragma once
+#include <cstdint>
 #include <thread>
 #include <vector>
 
@@ -23,6 +24,20 @@ void host_shares(int shares, const F &f)
     if (shares > 0) f(0);
     for (int t = started; t < shares; ++t) f(t);
     for (auto &x : th) x.join();
+}
+
+// The cell of each of n particles from the starts [ncell + 1] of an image that
+// may be damaged: false, and nothing written, unless they rise from 0 to n (a
+// start beyond n followed by smaller ones would have keys written past the
+// end).
+inline bool keys_of_starts(const int *starts, int ncell, int64_t n, int *key)
+{
+    if (starts[0] != 0 || starts[ncell] != n) return false;
+    for (int g = 0; g < ncell; ++g)
+        if (starts[g + 1] < starts[g]) return false;
+    for (int g = 0; g < ncell; ++g)
+        for (int k = starts[g]; k < starts[g + 1]; ++k) key[k] = g;
+    return true;
 }
 
 }  // namespace pic
